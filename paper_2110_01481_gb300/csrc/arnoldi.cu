@@ -514,10 +514,7 @@ sub_norm2_kernel(const float *a, const float *c, float *out, int64_t L,
 }
 
 // ---- batched kernels (one launch for every instance of a batch) ----------
-// map[blockIdx.x] = (instance, block of that instance).  The CGS2 passes take
-// kBatchFusedE float4 per thread, the slices of the one-launch step: the same
-// partial sums in the same order, so a solve's basis does not depend on which
-// of the two forms its step takes, bit for bit.
+// E = 1 passes; map[blockIdx.x] = (instance, block of that instance).
 
 __device__ __forceinline__ int vec_blocks_dev(long long L) {
     return (int)(((L + 3) / 4 + kThreads - 1) / kThreads);
@@ -534,8 +531,8 @@ batch_cgs_pass_kernel(BatchInst *__restrict__ insts, const int2 *__restrict__ ma
     float *q = I.variant == CTG_AB ? I.vm : I.vn;
     const double *coef = UPDATE ? (DOTS ? I.h1 : I.h2) : nullptr;
     double *red_out = DOTS ? (UPDATE ? I.h2 : I.h1) : I.scal + 1;
-    cgs_pass_body<T, kBatchFusedE, UPDATE, DOTS, NORM>(static_cast<const T *>(I.W), I.ldw, I.k, q, I.L, coef,
-                                                       I.partials, I.counter, red_out, mp.y, I.G);
+    cgs_pass_body<T, 1, UPDATE, DOTS, NORM>(static_cast<const T *>(I.W), I.ldw, I.k, q, I.L, coef,
+                                            I.partials, I.counter, red_out, mp.y, I.G);
 }
 
 // Last CGS2 pass and scaling of every instance (update_scale_body): the new
@@ -547,9 +544,9 @@ batch_update_scale_kernel(BatchInst *__restrict__ insts, const int2 *__restrict_
     BatchInst &I = insts[mp.x];
     if (!I.active) return;
     float *q = I.variant == CTG_AB ? I.vm : I.vn;
-    update_scale_body<T, kBatchFusedE>(static_cast<const T *>(I.W), I.ldw, I.k, q, I.L, I.h1, I.h2,
-                                       static_cast<T *>(I.W) + (size_t)I.k * I.ldw,
-                                       I.H + (size_t)(I.k - 1) * (I.maxit + 1), I.scal + 1, mp.y);
+    update_scale_body<T, 1>(static_cast<const T *>(I.W), I.ldw, I.k, q, I.L, I.h1, I.h2,
+                            static_cast<T *>(I.W) + (size_t)I.k * I.ldw,
+                            I.H + (size_t)(I.k - 1) * (I.maxit + 1), I.scal + 1, mp.y);
 }
 
 // One warp per instance: FP64 Givens update of the Hessenberg least-squares

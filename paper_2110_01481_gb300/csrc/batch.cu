@@ -98,7 +98,7 @@ size_t plan_instance(InstPlan &p, char *base) {
     d.L = L;
     d.maxit = maxit;
     d.ldw = (long long)ldw;
-    d.G = batch_fused_blocks(L);
+    d.G = ctg_vec_blocks(L);
     d.target = p.o.noise_norm > 0.0 ? p.o.tau * p.o.noise_norm : 0.0;
     d.wtype = p.o.basis_dtype;
     // the basis is the only O(maxit L) buffer: the storage law k L of Table 3
@@ -121,8 +121,8 @@ size_t plan_instance(InstPlan &p, char *base) {
     d.mt = g.back_model != CTG_BACK_PIXEL ? (const MatchedAngle *)take(sizeof(MatchedAngle) * g.n_angles)
                                           : nullptr;
     d.back_thr = 0.0f;
-    // partial rows: maxit + 3 rows of the passes, or 2 k + 2 rows of the fused
-    // step (k <= its largest k) over its blocks
+    // partial rows: maxit + 3 rows of the E = 1 passes, or 2 k + 2 rows of
+    // the fused step (k <= its largest k) over its blocks
     const int kf = maxit < ctg_batch_fused_max_k() ? maxit : ctg_batch_fused_max_k();
     const size_t rows_pass = (size_t)(maxit + 3) * Gp;
     const size_t rows_fused = (size_t)(2 * kf + 2) * padded4(batch_fused_blocks(L));
@@ -192,7 +192,7 @@ RedScratch scratch_of(const BatchInst &d) {
     rs.scal = d.scal;
     rs.counter = d.counter;
     rs.grid = d.G;
-    rs.E = kBatchFusedE;
+    rs.E = 1;
     return rs;
 }
 
@@ -243,11 +243,11 @@ void release(ctg_batch *b) {
 //     DP stop: x_k = x0 + W_k y_k; BA: stage w_{k+1} (and x_k), t_{k+1} =
 //     A w_{k+1} (and A x_k); BA with the DP stop: ||b - A x_k||; the
 //     stopping rules.
-// MB_CGS*: the blocks of the CGS2 passes and of the one-launch CGS2 step with
-// the Givens update (batch_fused_blocks per instance), which takes their place
-// and the separate Givens launch's while every step is at most fused_kcap.
+// MB_CGSF*: the blocks of the one-launch CGS2 step with the Givens update
+// (batch_fused_blocks per instance), used instead of MB_CGS* and the
+// separate Givens launch while every step is at most fused_kcap.
 enum { MB_BACK, MB_B16, MB_H16, MB_PAD_AB, MB_FWD_AB, MB_CGS, MB_CGS_B16, MB_CGS_H16,
-       MB_ITER, MB_PAD_BA, MB_FWD_BA, MB_RES, MB_COUNT };
+       MB_ITER, MB_PAD_BA, MB_FWD_BA, MB_RES, MB_CGSF, MB_CGSF_B16, MB_CGSF_H16, MB_COUNT };
 struct RoundSpec {
     BatchInst *insts;
     int n_inst;
@@ -323,8 +323,8 @@ void build_maps(const Plans &plans, const std::vector<int> &ids, std::vector<int
     add_fwd(MB_FWD_AB, true);
     auto cgs_blocks = [](const InstPlan &p, int wtype) {
         if (p.o.basis_dtype != wtype) return 0;
-        return batch_fused_blocks(p.variant == CTG_BA ? (long long)p.g.N * p.g.N
-                                                      : (long long)p.g.n_angles * p.g.n_det);
+        return ctg_vec_blocks(p.variant == CTG_BA ? (long long)p.g.N * p.g.N
+                                                  : (long long)p.g.n_angles * p.g.n_det);
     };
     add(MB_CGS, [&](const InstPlan &p) { return cgs_blocks(p, CTG_BASIS_FP32); });
     add(MB_CGS_B16, [&](const InstPlan &p) { return cgs_blocks(p, CTG_BASIS_BF16); });
@@ -335,6 +335,14 @@ void build_maps(const Plans &plans, const std::vector<int> &ids, std::vector<int
     add(MB_RES, [&](const InstPlan &p) {
         return ba_dp(p) ? ctg_vec_blocks((long long)p.g.n_angles * p.g.n_det) : 0;
     });
+    auto fused_blocks = [](const InstPlan &p, int wtype) {
+        if (p.o.basis_dtype != wtype) return 0;
+        return batch_fused_blocks(p.variant == CTG_BA ? (long long)p.g.N * p.g.N
+                                                      : (long long)p.g.n_angles * p.g.n_det);
+    };
+    add(MB_CGSF, [&](const InstPlan &p) { return fused_blocks(p, CTG_BASIS_FP32); });
+    add(MB_CGSF_B16, [&](const InstPlan &p) { return fused_blocks(p, CTG_BASIS_BF16); });
+    add(MB_CGSF_H16, [&](const InstPlan &p) { return fused_blocks(p, CTG_BASIS_FP16); });
 }
 
 // The largest k of the fused step for a batch whose maps are in rs (0 when
@@ -342,7 +350,7 @@ void build_maps(const Plans &plans, const std::vector<int> &ids, std::vector<int
 // then takes the separate passes throughout).
 int fused_kcap_of(const RoundSpec &rs, int max_maxit) {
     const int kcap = max_maxit < ctg_batch_fused_max_k() ? max_maxit : ctg_batch_fused_max_k();
-    const int which[3] = {MB_CGS, MB_CGS_B16, MB_CGS_H16};
+    const int which[3] = {MB_CGSF, MB_CGSF_B16, MB_CGSF_H16};
     const int types[3] = {CTG_BASIS_FP32, CTG_BASIS_BF16, CTG_BASIS_FP16};
     for (int t = 0; t < 3; ++t)
         if (rs.len[which[t]] > 0 && rs.len[which[t]] > ctg_batch_fused_resident(kcap, types[t])) return 0;
@@ -379,7 +387,7 @@ cudaError_t enqueue_round(const RoundSpec &r, cudaStream_t st, int *loop_ctl = n
     if (e == cudaSuccess)
         e = ctg_batch_forward(r.insts, map(MB_FWD_AB), r.len[MB_FWD_AB], CTG_AB, st, r.fwd_shape_ab);
     if (fused) {
-        const int which[3] = {MB_CGS, MB_CGS_B16, MB_CGS_H16};
+        const int which[3] = {MB_CGSF, MB_CGSF_B16, MB_CGSF_H16};
         const int types[3] = {CTG_BASIS_FP32, CTG_BASIS_BF16, CTG_BASIS_FP16};
         for (int t = 0; t < 3 && e == cudaSuccess; ++t)
             e = ctg_batch_cgs2_fused(r.insts, map(which[t]), r.len[which[t]], r.fused_kcap, r.bar, r.err, r.spin,

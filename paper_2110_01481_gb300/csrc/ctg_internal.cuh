@@ -405,7 +405,7 @@ struct BatchInst {
     const float *b;       // the solve's data b (m floats), start x0 (or NULL) and
     const float *x0;      // iterate x (n floats; BA with the DP stop forms x_k
     float *x;             // there every round)
-    // reduction scratch of this instance (kBatchFusedE float4 per thread, grid G)
+    // reduction scratch of this instance (E = 1 passes, grid G)
     float *partials;
     double *h1, *h2, *scal;
     unsigned *counter;
@@ -464,7 +464,7 @@ cudaError_t ctg_batch_finish_loop(BatchInst *insts, int n_inst, int *ctl, int ma
                                   cudaGraphConditionalHandle h_next = 0, int fused_max = 0);
 // Exit: y = R^{-1} g for the instance's final k.
 cudaError_t ctg_batch_solve_y(BatchInst *insts, int n_inst, int max_k, cudaStream_t st);
-int ctg_vec_blocks(long long L);          // blocks of a vector pass over L with one float4 per thread
+int ctg_vec_blocks(long long L);          // blocks of an E = 1 vector pass over L
 
 // The batched one-launch CGS2 step with each instance's Givens update
 // (steps k <= ctg_batch_fused_max_k()): kBatchFusedE float4 groups per
