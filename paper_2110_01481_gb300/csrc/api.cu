@@ -147,6 +147,7 @@ struct GeomEntry {
     FwdAngle *fwd = nullptr;
     BackAngle *back = nullptr;
     int back_window = 0;        // detector window of the tiled back projector
+    bool back_blocks = false;   // the pixel-driven B takes 2 x 2 pixel blocks
     PadLayout pl{};             // staged-image layout of the forward projector
     float2 *pad = nullptr;      // context-owned staged image for ctg_project
     float2 *tw = nullptr;       // NCP: DFT twiddles of length n_det (on first use)
@@ -172,8 +173,8 @@ cudaError_t back_apply(const GeomEntry *ge, const void *b, int btype, const floa
                        cudaStream_t st, ColRef bc = col_none()) {
     const ctg_geom *g = &ge->g;
     if (g->back_model == CTG_BACK_PIXEL)
-        return ctg_launch_back(b, btype, g->N, g->n_angles, g->n_det, ge->back, ge->back_window, add,
-                               x, st, ge->back_chunk, bc);
+        return ctg_launch_back(b, btype, g->N, g->n_angles, g->n_det, ge->back, ge->back_window,
+                               ge->back_blocks, add, x, st, ge->back_chunk, bc);
     if (ge->rm == 0 && ge->back_window <= ctg_back_window_max())
         return ctg_launch_back_matched_tiled(b, btype, g->N, g->n_angles, g->n_det, ge->back,
                                              ge->back_window, ge->mt, ge->thr, add, x, st, bc);
@@ -402,7 +403,7 @@ int tune_geometry(GeomEntry *ge) {
             timed([&] {
                 if (err == cudaSuccess)
                     err = ctg_launch_back(bv, CTG_BASIS_FP32, g->N, g->n_angles, g->n_det, ge->back,
-                                          ge->back_window, nullptr, xv, st, back_cand[c]);
+                                          ge->back_window, ge->back_blocks, nullptr, xv, st, back_cand[c]);
             }, &ge->back_us[c]);
     if (err == cudaSuccess) {
         int fs = 0;
@@ -489,6 +490,7 @@ int get_geom(ctg_ctx *ctx, const ctg_geom *g, GeomEntry **out) {
     e.last_use = ++ctx->tick;
     e.serial = e.last_use;
     e.back_window = ctg_back_window(bk.data(), g->n_angles);
+    e.back_blocks = ctg_back_blocks_ok(bk.data(), g->n_angles);
     e.pl = ctg_pad_layout(g->N, g->det_spacing);
     cudaError_t err = cudaMalloc(&e.fwd, sizeof(FwdAngle) * fw.size());
     if (err == cudaSuccess) err = cudaMalloc(&e.back, sizeof(BackAngle) * bk.size());

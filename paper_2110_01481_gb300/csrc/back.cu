@@ -1,0 +1,682 @@
+// The back projectors of single launches: the pixel-driven B (paper Sec. 1,
+// eq. (1.2)), the matched A^T and the thresholded B_tau of Sec. 6.5, gather-only
+// (no atomics).
+#include <cooperative_groups.h>
+
+#include <algorithm>
+#include <type_traits>
+
+#include "proj_device.cuh"
+
+namespace cg = cooperative_groups;
+
+namespace {
+
+// ---- one pixel and its reflection: A^T, B_tau, and B for pitches below a pixel ----
+// Image grid and detector are centred, so pixel
+// (i, j) and its point reflection (N-1-i, N-1-j) sit at detector positions u
+// and (n_det-1) - u of every angle: with the reversed projection b'[d] =
+// b[n_det-1-d] the reflected pixel interpolates b' at the same u, with the
+// same index and weight.  So a tile covers 32 x 32 pixels of the upper half of
+// the image and their reflections: position, floor, weight and shared address
+// are formed once for two interpolations, and one 16-byte shared load brings
+// the operands of both.
+//
+// A thread-block cluster of kSplit CTAs owns a tile; each CTA sums a contiguous
+// share of the angles.  For a chunk of angles a CTA stages, per angle, the
+// detector window that the tile projects onto as (b[d], b'[d], b[d+1] - b[d],
+// b'[d+1] - b'[d]) in shared memory (zeros outside the detector), so the inner
+// loop has no bounds test.  The tile centre's detector position is formed
+// exactly in fixed point; each pixel adds a float offset of at most 22
+// bins.  The CTAs' partial sums are then added through distributed shared
+// memory in rank order (deterministic, no atomics), each CTA finishing a share
+// of the tile's rows.
+// Bound by the shared-memory data path (8 bytes per interpolation, 16 per clock
+// and SM; 2048^2, 1800 angles run at 80 % of that): the pixel-driven B at 512^2,
+// 720 angles takes 63 us and at 2048^2 1,908 us, against 73 and 2,381 us with one
+// pixel per position.
+constexpr int kPT = 32;             // tile side
+constexpr int kPairRows = 8;        // rows per thread (threads: 32 x 4): the shared parameter load and the
+                                    // address base of an angle serve 16 interpolations (512^2, 720 angles:
+                                    // 63 us against 67 with 4 rows and 256 threads)
+constexpr int kPairThreads = 128;
+template <int kRows>
+__host__ __device__ constexpr int pair_threads() { return kPT * (kPT / kRows); }
+constexpr int kPairChunk = 32;      // angles staged per pass
+constexpr int kPairSplit = 8;       // CTAs per cluster = angle groups per tile (512^2: 63 us, 76 us with 4)
+// tiles of an image: columns x rows of the upper half
+__host__ __device__ constexpr int back_tiles_x(int N) { return (N + kPT - 1) / kPT; }
+__host__ __device__ constexpr int back_tiles_y(int N) { return ((N + 1) / 2 + kPT - 1) / kPT; }
+
+__device__ __forceinline__ void add2(float &a0, float &a1, float v0, float v1) {
+    asm("{\n\t.reg .b64 a, v;\n\t"
+        "mov.b64 a, {%0, %1};\n\t"
+        "mov.b64 v, {%2, %3};\n\t"
+        "add.rn.f32x2 a, a, v;\n\t"
+        "mov.b64 {%0, %1}, a;\n\t}"
+        : "+f"(a0), "+f"(a1)
+        : "f"(v0), "f"(v1));
+}
+
+// Body of one CTA of the back-projection cluster for tile (bx, by).  Every
+// CTA of a cluster must call it (it synchronises the cluster twice).
+// kModel: 0 the pixel-driven B (linear interpolation on the detector);
+// 1 the matched A^T and 2 the thresholded B_tau, whose weights for the two
+// nearest bins d0, d0 + 1 of a pixel at detector position d0 + f are
+// scale * max(0, 1 - f inv_w) and scale * max(0, 1 - (1 - f) inv_w) (terms
+// below thr dropped for 2).  The staged entries are (b[d], b'[d], differences)
+// for the pixel-driven B and (b[d], b'[d], b[d+1], b'[d+1]) for the others.
+// kRows: pixel rows per thread, kPT / kRows row threads per column (rows
+// di, di + kPT / kRows, ...).
+template <typename T, int kModel = 0, int kChunk = kPairChunk, int kRows = kPairRows, int kSplit = kPairSplit>
+__device__ __forceinline__ void pixel_pair_tile(const T *__restrict__ b, int N, int n_angles,
+                                                int n_det, const BackAngle *__restrict__ tab,
+                                                int W, const float *__restrict__ add,
+                                                float *__restrict__ x, int bx, int by,
+                                                const MatchedAngle *__restrict__ mt = nullptr,
+                                                float thr = 0.0f) {
+    constexpr int kThr = pair_threads<kRows>(), kRT = kPT / kRows;
+    static_assert(kChunk <= kThr && kRows % 2 == 0 && kRows <= 16, "back tile shape");
+    extern __shared__ float4 s_win[];                 // kChunk * W entries; at the end the partial sums
+    __shared__ float4 s_par[kChunk];                  // cf, sf, u at the tile centre, kRT sf
+    __shared__ int s_org[kChunk];                     // detector bin of the window's first entry
+    __shared__ float4 s_wt[kModel ? kChunk : 1];      // scale, scale inv_w, scale - scale inv_w
+    float *s_part = reinterpret_cast<float *>(s_win); // [2 kRows][kThr]
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank();       // == blockIdx.z
+    const int j0 = bx * kPT, i0 = by * kPT;
+    const int dj = threadIdx.x & 31, di = threadIdx.x >> 5;   // di in [0, kRT)
+    const float fdj = (float)dj - 0.5f * (kPT - 1), fdi = (float)di - 0.5f * (kPT - 1);
+    const int per = (n_angles + kSplit - 1) / kSplit;
+    const int a_begin = min(n_angles, rank * per), a_end = min(n_angles, a_begin + per);
+    const int wc = W / 2;                             // window entry of the tile centre's bin
+    float acc[kRows][2];                              // direct and reflected pixel
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) acc[r][0] = acc[r][1] = 0.f;
+    for (int a0 = a_begin; a0 < a_end; a0 += kChunk) {
+        const int na = min(kChunk, a_end - a0);
+        __syncthreads();
+        if (threadIdx.x < na) {
+            const BackAngle t = tab[a0 + threadIdx.x];
+            // the tile centre is 15.5 pixels from its origin in both directions
+            const long long Uc = t.C + (long long)j0 * t.COS + (long long)i0 * t.SIN +
+                                 (((kPT - 1) * (t.COS + t.SIN)) >> 1);
+            s_par[threadIdx.x] = make_float4(t.cf, t.sf, fx_frac(Uc), (float)kRT * t.sf);
+            s_org[threadIdx.x] = (int)(Uc >> CTG_FX_BITS) - wc;
+            if constexpr (kModel != 0) {
+                const MatchedAngle m = mt[a0 + threadIdx.x];
+                const float sw = m.scale * m.inv_w;
+                s_wt[threadIdx.x] = make_float4(m.scale, sw, m.scale - sw, 0.0f);
+            }
+        }
+        __syncthreads();
+        // one warp per staged angle, lanes along its window (no division)
+        for (int k = threadIdx.x >> 5; k < na; k += kThr / 32) {
+            const int org = s_org[k];
+            const T *brow = b + (size_t)(a0 + k) * n_det;
+            float4 *dst = s_win + k * W;
+            auto bin = [&](int d) {
+                return ((unsigned)d < (unsigned)n_det) ? to_f(__ldg(brow + d)) : 0.0f;
+            };
+            for (int w = threadIdx.x & 31; w < W; w += 32) {
+                const int d = org + w, e = n_det - 1 - d;
+                const float v0 = bin(d), v1 = bin(d + 1), m0 = bin(e), m1 = bin(e - 1);
+                dst[w] = kModel == 0 ? make_float4(v0, m0, v1 - v0, m1 - m0) : make_float4(v0, m0, v1, m1);
+            }
+        }
+        __syncthreads();
+        // shared address of an angle's window centre less the magic number's
+        // bits times 16, so that row r's entry is at sb + 16 t_r (32-bit
+        // wrap-around) with t_r the bits of u_r + M: one shift-add per address
+        unsigned sb = (unsigned)__cvta_generic_to_shared(s_win + wc) - (0x4B400000u << 4);
+#pragma unroll 2
+        for (int k = 0; k < na; ++k, sb += 16u * (unsigned)W) {
+            const float4 p = s_par[k];
+            float u[kRows];
+            u[0] = fmaf(fdi, p.y, fmaf(fdj, p.x, p.z));
+#pragma unroll
+            for (int r = 1; r < kRows; ++r) u[r] = u[r - 1] + p.w;
+            float tt[kRows], ff[kRows];
+#pragma unroll
+            for (int r = 0; r < kRows; r += 2) floor_frac2(u[r], u[r + 1], tt[r], tt[r + 1], ff[r], ff[r + 1]);
+            float4 wt = make_float4(0.f, 0.f, 0.f, 0.f);
+            if constexpr (kModel != 0) wt = s_wt[k];
+#pragma unroll
+            for (int r = 0; r < kRows; ++r) {
+                const float f = ff[r];
+                const float4 e =
+                    *static_cast<const float4 *>(__cvta_shared_to_generic(sb + (__float_as_uint(tt[r]) << 4)));
+                if constexpr (kModel == 0) {
+                    add2(acc[r][0], acc[r][1], fmaf(f, e.z, e.x), fmaf(f, e.w, e.y));
+                } else {
+                    float w0 = fmaxf(0.0f, fmaf(-f, wt.y, wt.x));
+                    float w1 = fmaxf(0.0f, fmaf(f, wt.y, wt.z));
+                    if constexpr (kModel == 2) {
+                        w0 = w0 >= thr ? w0 : 0.0f;
+                        w1 = w1 >= thr ? w1 : 0.0f;
+                    }
+                    acc[r][0] = fmaf(w0, e.x, fmaf(w1, e.z, acc[r][0]));
+                    acc[r][1] = fmaf(w0, e.y, fmaf(w1, e.w, acc[r][1]));
+                }
+            }
+        }
+    }
+    __syncthreads();                                  // the windows have been read
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+        s_part[(2 * r) * kThr + threadIdx.x] = acc[r][0];
+        s_part[(2 * r + 1) * kThr + threadIdx.x] = acc[r][1];
+    }
+    cluster.sync();
+    // this CTA finishes planes rank, rank + kSplit, ...: plane 2 r + h holds
+    // pixel rows di + kRT r (h = 0) or their reflections (h = 1).  A pixel at
+    // or before the image's centre is written by the direct plane, the others
+    // by the reflected one (on the middle row of an odd N both reach it).
+    const long long last = (long long)N * N - 1;
+#pragma unroll
+    for (int q = rank; q < 2 * kRows; q += kSplit) {
+        float sum = 0.0f;
+#pragma unroll
+        for (int c = 0; c < kSplit; ++c) sum += cluster.map_shared_rank(s_part + q * kThr, c)[threadIdx.x];
+        const int i = i0 + di + kRT * (q >> 1), j = j0 + dj;
+        const long long p = (long long)i * N + j;
+        if (i < N && j < N && ((q & 1) ? 2 * p < last : 2 * p <= last)) {
+            const long long o = (q & 1) ? last - p : p;
+            x[o] = add ? sum + add[o] : sum;
+        }
+    }
+    cluster.sync();   // peers' shared memory must outlive the reads above
+}
+
+// ---- 2 x 2 pixel blocks: the pixel-driven B for pitches of a pixel or more ----
+// One interpolation per shared load is bound by the shared-memory data path
+// (8 bytes per interpolation, 16 interpolations per clock and SM).  Where one
+// pixel step moves at most one detector bin (|cos|, |sin| <= the pitch), a 2 x 2
+// block of pixels lies within [v, v + 1.42] bins of its lowest corner, so four
+// bins b0..b3 from floor(v) on serve all four pixels (and four reversed ones
+// their reflections): 4 bytes per interpolation, and one floor and one address
+// for eight.  With D = b1 - b0, K1 and K2 the second differences at b1 and b2, f
+// the corner's fraction and oB, oC the block's steps along its columns and rows,
+// the interpolant at f + o is
+//   b0 + D f + D o + K1 max(0, f + o - 1) + K2 max(0, f + o - 2),
+// so over the angles the four pixels share the sums S = sum (b0 + D f), G =
+// sum D oB, H = sum D oC: corner S, next column B = S + G + sum K1 r1(oB), next
+// row C = S + H + sum K1 r1(oC), far corner E = S + G + H + sum (K1 r1(oB + oC) +
+// K2 r2(oB + oC)) (K2 enters only there, as oB, oC <= 1).
+// An angle with sin < 0 is taken as its opposite (the reversed projection), so
+// the lowest corner is the left column for cos >= 0 and the right one for cos
+// < 0; the sums go to the pixels when that changes, and every kBlkFlush chunks
+// (which also keeps the chains of additions short: at 512^2, 720 angles the error
+// against FP64 is 6.6e-8 on smooth data and 7.4e-7 on white noise, 0.6 and 0.4
+// times that of one pixel per position from the tile's corner).
+// The raw bins are staged by 4-byte cp.async (rows have any alignment) one chunk
+// ahead.  Now bound by issue slots and the FMA pipe (about 4 issued instructions
+// per interpolation, 70 % of the slots): 512^2, 720 angles 73 -> 49 us (3.8 T
+// interpolations/s), 2048^2, 1800 angles 2,381 -> 1,399 us (5.4 T/s).
+constexpr int kBlkWarps = 4, kBlkThreads = 32 * kBlkWarps;
+constexpr int kBlkChunk = 16;         // angles per stage, two stages in flight
+constexpr int kBlkFlush = 4;
+// Window of a 32 x th tile: a block's lowest corner lies within half the tile's
+// diagonal of the centre (21.92 bins for 32 rows, 35.11 for 64) plus a phase below
+// one, and reads the three bins after its own.
+constexpr int blk_centre(int th) { return th <= 32 ? 24 : 37; }
+constexpr int blk_window(int th) { return th <= 32 ? 52 : 78; }
+
+__device__ __forceinline__ float sat_add(float a, float b) { return __saturatef(a + b); }
+
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
+    float2 r;
+    asm("{\n\t.reg .b64 a, b, r;\n\t"
+        "mov.b64 a, {%2, %3};\n\t"
+        "mov.b64 b, {%4, %5};\n\t"
+        "sub.rn.f32x2 r, a, b;\n\t"
+        "mov.b64 {%0, %1}, r;\n\t}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+// acc += a * (s, s)
+__device__ __forceinline__ void fma2s(float2 &acc, float2 a, float s) {
+    asm("{\n\t.reg .b64 c, a, s;\n\t"
+        "mov.b64 c, {%0, %1};\n\t"
+        "mov.b64 a, {%2, %3};\n\t"
+        "mov.b64 s, {%4, %4};\n\t"
+        "fma.rn.f32x2 c, a, s, c;\n\t"
+        "mov.b64 {%0, %1}, c;\n\t}"
+        : "+f"(acc.x), "+f"(acc.y)
+        : "f"(a.x), "f"(a.y), "f"(s));
+}
+__device__ __forceinline__ void fma_each(float2 &acc, float2 a, float s) {
+    acc.x = fmaf(a.x, s, acc.x);
+    acc.y = fmaf(a.y, s, acc.y);
+}
+
+// The CTA's pixel sums for angles [a_begin, a_end) one interpolation at a time,
+// from global memory: taken when the block sums hold a value that is not
+// finite, because a second difference would carry an infinite or NaN bin (or
+// the overflow of a difference) to neighbours that do not interpolate it.
+template <typename T>
+__device__ __noinline__ void pixel_back_plain(const T *__restrict__ b, int n_det, const BackAngle *__restrict__ tab,
+                                              int a_begin, int a_end, int j0, int i0, int rows, float *s_px) {
+    for (int e = threadIdx.x; e < 2 * rows * kPT; e += blockDim.x) {
+        const int h = e / (rows * kPT), i = i0 + (e / kPT) % rows, j = j0 + e % kPT;
+        float acc = 0.0f;
+        for (int a = a_begin; a < a_end; ++a) {
+            const BackAngle t = tab[a];
+            const long long U = t.C + (long long)j * t.COS + (long long)i * t.SIN;
+            const int d = (int)(U >> CTG_FX_BITS), d0 = h ? n_det - 1 - d : d, d1 = h ? d0 - 1 : d0 + 1;
+            const float v0 = (unsigned)d0 < (unsigned)n_det ? to_f(__ldg(b + (size_t)a * n_det + d0)) : 0.0f;
+            const float v1 = (unsigned)d1 < (unsigned)n_det ? to_f(__ldg(b + (size_t)a * n_det + d1)) : 0.0f;
+            acc += fmaf(fx_frac(U), v1 - v0, v0);
+        }
+        s_px[e] = acc;
+    }
+}
+
+// Body of one CTA of the cluster for the 32 x (16 kNB) tile (bx, by) of the
+// upper half; each of the 128 threads owns kNB blocks 16 rows apart.  Every CTA
+// of a cluster must call it.
+template <typename T, int kNB, int kSplit = kPairSplit>
+__device__ __forceinline__ void pixel_back_blocks(const T *__restrict__ b, int N, int n_angles, int n_det,
+                                                  const BackAngle *__restrict__ tab,
+                                                  const float *__restrict__ add, float *__restrict__ x, int bx,
+                                                  int by) {
+    constexpr int kThr = kBlkThreads, kStep = 4 * kBlkWarps, kTH = kStep * kNB;   // rows between blocks; tile height
+    constexpr int kWin = blk_window(kTH), kCentre = blk_centre(kTH);
+    extern __shared__ float4 s_dyn[];
+    float2 *s_win = reinterpret_cast<float2 *>(s_dyn);            // [2][kBlkChunk][kWin] (b, b')
+    float *s_px = reinterpret_cast<float *>(s_win + 2 * kBlkChunk * kWin);   // [2][kTH][32] sums of the pixels
+    static_assert(kNB % 2 == 0 && kTH <= 64, "block tile shape");
+    // per angle: phase at the tile centre, oB, oC, oB - 1; oC - 1, oB + oC - 1, oB + oC - 2
+    __shared__ float4 s_par[4][kBlkChunk][2];
+    __shared__ int2 s_org[4][kBlkChunk];                          // first bin, flip
+    __shared__ unsigned s_right[4];                               // angles whose lowest corner is on the right
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int j0 = bx * kPT, i0 = by * kTH;
+    // a quarter warp holds 4 x 2 blocks, a warp 8 x 4 (16 x 8 pixels): the
+    // bins of a half warp's loads span at most 16 entries, no bank conflicts
+    const int cb = 8 * (warp & 1) + (lane & 3) + 4 * ((lane >> 3) & 1);
+    const int rb = 4 * (warp >> 1) + ((lane >> 2) & 1) + 2 * (lane >> 4);
+    const float fdj = 2.0f * cb - 0.5f * (kPT - 1), fdi = 2.0f * rb - 0.5f * (kTH - 1);
+    const int per = (n_angles + kSplit - 1) / kSplit;
+    const int a_begin = min(n_angles, rank * per), a_end = min(n_angles, a_begin + per);
+    const int nchunks = (a_end - a_begin + kBlkChunk - 1) / kBlkChunk;
+    for (int e = tid; e < 2 * kTH * kPT / 4; e += kThr)
+        reinterpret_cast<float4 *>(s_px)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+
+    auto params = [&](int c) {
+        if (warp != 0) return;
+        const int k = lane, a = a_begin + c * kBlkChunk + k;
+        bool right = false;
+        if (k < kBlkChunk && a < a_end) {
+            const BackAngle t = tab[a];
+            long long Uc = t.C + (long long)j0 * t.COS + (long long)i0 * t.SIN +
+                           (((kPT - 1) * t.COS + (kTH - 1) * t.SIN) >> 1);
+            float cf = t.cf, sf = t.sf;
+            const int flip = t.SIN < 0;
+            if (flip) {
+                Uc = ((long long)(n_det - 1) << CTG_FX_BITS) - Uc;
+                cf = -cf;
+                sf = -sf;
+            }
+            right = cf < 0.0f;
+            const float oB = fabsf(cf);
+            s_par[c & 3][k][0] = make_float4(fx_frac(Uc), oB, sf, oB - 1.0f);
+            s_par[c & 3][k][1] = make_float4(sf - 1.0f, oB + (sf - 1.0f), (oB - 1.0f) + (sf - 1.0f), 0.0f);
+            s_org[c & 3][k] = make_int2((int)(Uc >> CTG_FX_BITS) - kCentre, flip);
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, right);
+        if (lane == 0) s_right[c & 3] = m;
+    };
+    auto stage = [&](int c) {
+        const int a0 = a_begin + c * kBlkChunk, na = min(kBlkChunk, a_end - a0);
+        for (int k = warp; k < na; k += kBlkWarps) {
+            const int2 o = s_org[c & 3][k];
+            const T *row = b + (size_t)(a0 + k) * n_det;
+            float2 *dst = s_win + ((c & 1) * kBlkChunk + k) * kWin;
+            for (int w = lane; w < kWin; w += 32) {
+                const int d = o.x + w, e = n_det - 1 - d;
+                const bool in = (unsigned)d < (unsigned)n_det;     // e is in range exactly when d is
+                const T *p0 = row + (in ? (o.y ? e : d) : 0), *p1 = row + (in ? (o.y ? d : e) : 0);
+                if constexpr (std::is_same<T, float>::value) {
+                    const unsigned s0 = (unsigned)__cvta_generic_to_shared(dst + w);
+                    const int sz = in ? 4 : 0;
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(s0), "l"(p0), "r"(sz));
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(s0 + 4), "l"(p1), "r"(sz));
+                } else {
+                    dst[w] = in ? make_float2(to_f(__ldg(p0)), to_f(__ldg(p1))) : make_float2(0.f, 0.f);
+                }
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+
+    float2 S[kNB], G[kNB], H[kNB], B[kNB], C[kNB], E[kNB];
+    auto clear = [&] {
+#pragma unroll
+        for (int q = 0; q < kNB; ++q) S[q] = G[q] = H[q] = B[q] = C[q] = E[q] = make_float2(0.f, 0.f);
+    };
+    auto flush = [&](bool right) {
+#pragma unroll
+        for (int q = 0; q < kNB; ++q) {
+            const int row = 2 * rb + kStep * q, col = 2 * cb;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                auto at = [&](const float2 &v) { return h ? v.y : v.x; };
+                const float a = at(S[q]), bb = (at(S[q]) + at(G[q])) + at(B[q]);
+                const float cc = (at(S[q]) + at(H[q])) + at(C[q]);
+                const float ee = (at(S[q]) + (at(G[q]) + at(H[q]))) + at(E[q]);
+                float2 *p0 = reinterpret_cast<float2 *>(s_px + (h * kTH + row) * kPT + col);
+                float2 *p1 = reinterpret_cast<float2 *>(s_px + (h * kTH + row + 1) * kPT + col);
+                float2 t0 = *p0, t1 = *p1;
+                t0.x += right ? bb : a;
+                t0.y += right ? a : bb;
+                t1.x += right ? ee : cc;
+                t1.y += right ? cc : ee;
+                *p0 = t0;
+                *p1 = t1;
+            }
+        }
+        clear();
+    };
+    clear();
+    bool right = false;
+    float sdj = fdj;                        // u = phase + oB sdj + oC fdi at the block's lowest corner
+    params(0);
+    __syncthreads();
+    stage(0);
+    for (int c = 0; c < nchunks; ++c) {
+        if (c + 1 < nchunks) params(c + 1); // (slower warps may still read those of c - 1 and c)
+        __syncthreads();                    // params of c + 1 written; the windows of c - 1 have been read
+        if (c + 1 < nchunks) {
+            stage(c + 1);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();                    // the windows of c have landed
+        const int na = min(kBlkChunk, a_end - a_begin - c * kBlkChunk);
+        const float4 (*par)[2] = s_par[c & 3];
+        // shared address of the window's centre less the magic number's bits
+        // times 8 (32-bit wrap-around), as in pixel_pair_tile
+        unsigned sb = (unsigned)__cvta_generic_to_shared(s_win + (c & 1) * kBlkChunk * kWin + kCentre) -
+                      (0x4B400000u << 3);
+        // runs of angles with the lowest corner on the same side
+        const unsigned rights = s_right[c & 3];
+        for (int k = 0; k < na;) {
+            const bool r = (rights >> k) & 1;
+            const unsigned change = (r ? ~rights : rights) >> k;
+            const int end = change ? min(na, k + __ffs(change) - 1) : na;
+            if (r != right) {
+                flush(right);
+                right = r;
+                sdj = r ? -(fdj + 1.0f) : fdj;
+            }
+#pragma unroll 2
+            for (; k < end; ++k, sb += 8u * kWin) {
+                const float4 p = par[k][0], o = par[k][1];
+                const float u0 = fmaf(p.z, fdi, fmaf(p.y, sdj, p.x));
+                float tt[kNB], ff[kNB];
+#pragma unroll
+                for (int q = 0; q < kNB; q += 2)
+                    floor_frac2(fmaf(p.z, (float)(kStep * q), u0), fmaf(p.z, (float)(kStep * (q + 1)), u0), tt[q],
+                                tt[q + 1], ff[q], ff[q + 1]);
+#pragma unroll
+                for (int q = 0; q < kNB; ++q) {
+                    const unsigned at = sb + (__float_as_uint(tt[q]) << 3);
+                    const float2 *e = static_cast<const float2 *>(__cvta_shared_to_generic(at));
+                    const float2 b0 = e[0], b1 = e[1], b2 = e[2], b3 = e[3];
+                    const float f = ff[q];
+                    const float2 D0 = sub2(b1, b0), D1 = sub2(b2, b1), D2 = sub2(b3, b2);
+                    const float2 K1 = sub2(D1, D0), K2 = sub2(D2, D1);
+                    add2(S[q].x, S[q].y, b0.x, b0.y);
+                    fma_each(S[q], D0, f);
+                    fma2s(G[q], D0, p.y);
+                    fma2s(H[q], D0, p.z);
+                    fma_each(B[q], K1, sat_add(f, p.w));
+                    fma_each(C[q], K1, sat_add(f, o.x));
+                    fma_each(E[q], K1, fmaxf(f + o.y, 0.0f));
+                    fma_each(E[q], K2, sat_add(f, o.z));
+                }
+            }
+        }
+        if (c % kBlkFlush == kBlkFlush - 1) flush(right);
+    }
+    flush(right);
+    {
+        bool bad = false;
+#pragma unroll
+        for (int q = 0; q < kNB; ++q)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const float2 v = *reinterpret_cast<const float2 *>(
+                    s_px + ((r >> 1) * kTH + 2 * rb + kStep * q + (r & 1)) * kPT + 2 * cb);
+                bad = bad || !(fabsf(v.x) <= 3.402823466e38f) || !(fabsf(v.y) <= 3.402823466e38f);
+            }
+        if (__syncthreads_or(bad)) pixel_back_plain<T>(b, n_det, tab, a_begin, a_end, j0, i0, kTH, s_px);
+    }
+    cluster.sync();
+    // this CTA finishes a share of the 2 x (kTH x 32) sums: h = 0 the tile's
+    // pixels, h = 1 their reflections.  A pixel at or before the image's centre
+    // is written by h = 0, the others by h = 1 (on the middle row of an odd N
+    // both reach it).
+    const long long last = (long long)N * N - 1;
+    constexpr int kShare = 2 * kTH * kPT / kSplit;
+    for (int e = rank * kShare + tid; e < (rank + 1) * kShare; e += kThr) {
+        float sum = 0.0f;
+#pragma unroll
+        for (int q = 0; q < kSplit; ++q) sum += cluster.map_shared_rank(s_px, q)[e];
+        const int h = e / (kTH * kPT), i = i0 + (e / kPT) % kTH, j = j0 + e % kPT;
+        const long long p = (long long)i * N + j;
+        if (i < N && j < N && (h ? 2 * p < last : 2 * p <= last)) {
+            const long long o = h ? last - p : p;
+            x[o] = add ? sum + add[o] : sum;
+        }
+    }
+    cluster.sync();   // peers' shared memory must outlive the reads above
+}
+constexpr size_t blk_smem(int nb) {
+    return sizeof(float2) * 2 * kBlkChunk * blk_window(16 * nb) + sizeof(float) * 2 * 16 * nb * kPT;
+}
+// Blocks per thread for an image: four (64-row tiles, half the staging and
+// parameter loads per pixel) once that leaves about three CTAs per SM, else two
+// (512^2: 49 against 51.5 us, 2048^2: 1,399 against 1,489; 361^2: 14.2 against 12.5).
+constexpr int blk_tiles_y(int N, int nb) { return ((N + 1) / 2 + 16 * nb - 1) / (16 * nb); }
+constexpr int blk_nb(int N) { return back_tiles_x(N) * blk_tiles_y(N, 4) * kPairSplit >= 456 ? 4 : 2; }
+
+template <typename T, int kNB>
+__global__ void __cluster_dims__(1, 1, kPairSplit) __launch_bounds__(kBlkThreads, kNB == 4 ? 4 : 7)
+pixel_back_blocks_kernel(const T *__restrict__ b, ColRef bc, int N, int n_angles, int n_det,
+                         const BackAngle *__restrict__ tab, const float *__restrict__ add, float *__restrict__ x) {
+    pixel_back_blocks<T, kNB>(b + col_offset(bc), N, n_angles, n_det, tab, add, x, blockIdx.x, blockIdx.y);
+}
+
+// bc: the input is column bc of a basis (b + col_offset(bc)), or b itself.
+template <typename T, int kChunk>
+__global__ void __cluster_dims__(1, 1, kPairSplit) __launch_bounds__(kPairThreads)
+pixel_back_tiled_kernel(const T *__restrict__ b, ColRef bc, int N, int n_angles, int n_det,
+                        const BackAngle *__restrict__ tab, int W, const float *__restrict__ add,
+                        float *__restrict__ x) {
+    pixel_pair_tile<T, 0, kChunk, kPairRows>(b + col_offset(bc), N, n_angles, n_det, tab, W, add, x,
+                                               blockIdx.x, blockIdx.y);
+}
+
+// A^T (kModel 1) or B_tau (kModel 2) with the tiled design above.
+template <typename T, int kModel, int kChunk>
+__global__ void __cluster_dims__(1, 1, kPairSplit) __launch_bounds__(kPairThreads)
+matched_back_tiled_kernel(const T *__restrict__ b, ColRef bc, int N, int n_angles, int n_det,
+                          const BackAngle *__restrict__ tab, int W, const MatchedAngle *__restrict__ mt,
+                          float thr, const float *__restrict__ add, float *__restrict__ x) {
+    pixel_pair_tile<T, kModel, kChunk>(b + col_offset(bc), N, n_angles, n_det, tab, W, add, x, blockIdx.x, blockIdx.y,
+                               mt, thr);
+}
+
+// Generic pixel-driven back projection (any detector pitch): 32 x 8 tiles,
+// taps read through L1 with bounds tests.
+constexpr int kBX = 32, kBY = 8, kAChunk = 256;
+
+template <typename T>
+__global__ void __launch_bounds__(kBX *kBY)
+pixel_back_kernel(const T *__restrict__ b, ColRef bc, int N, int n_angles, int n_det,
+                  const BackAngle *__restrict__ tab, const float *__restrict__ add,
+                  float *__restrict__ x) {
+    __shared__ float4 sp[kAChunk];
+    b += col_offset(bc);
+    const int j0 = blockIdx.x * kBX, i0 = blockIdx.y * kBY;
+    const int dj = threadIdx.x, di = threadIdx.y;
+    const int tid = di * kBX + dj;
+    const float fdj = (float)dj, fdi = (float)di;
+    float acc = 0.0f;
+    for (int a0 = 0; a0 < n_angles; a0 += kAChunk) {
+        const int na = min(kAChunk, n_angles - a0);
+        __syncthreads();
+        if (tid < na) {
+            const BackAngle t = tab[a0 + tid];
+            const long long U0 = t.C + (long long)j0 * t.COS + (long long)i0 * t.SIN;
+            sp[tid] = make_float4(t.cf, t.sf, fx_frac(U0),
+                                  __int_as_float((int)(U0 >> CTG_FX_BITS)));
+        }
+        __syncthreads();
+        const T *brow = b + (size_t)a0 * n_det;
+#pragma unroll 4
+        for (int k = 0; k < na; ++k, brow += n_det) {
+            const float4 p = sp[k];
+            const float u = fmaf(fdi, p.y, fmaf(fdj, p.x, p.z));
+            const float fl = floorf(u);
+            const int dd = __float_as_int(p.w) + (int)fl;
+            const float f = u - fl;
+            const float v0 = ((unsigned)dd < (unsigned)n_det) ? to_f(__ldg(brow + dd)) : 0.0f;
+            const float v1 = ((unsigned)(dd + 1) < (unsigned)n_det) ? to_f(__ldg(brow + dd + 1)) : 0.0f;
+            acc += fmaf(f, v1 - v0, v0);
+        }
+    }
+    const int i = i0 + di, j = j0 + dj;
+    if (i < N && j < N) {
+        const size_t p = (size_t)i * N + j;
+        x[p] = add ? acc + add[p] : acc;
+    }
+}
+
+}  // namespace
+
+namespace {
+// Dynamic shared memory of the tiled back projectors: the staged windows (kept
+// to 40 KB, so that no launch needs an opt-in), or the partial sums that take
+// their place.
+constexpr size_t kBackSmem = 40 * 1024;
+constexpr int kPairChunkMin = 8;
+constexpr int kBackWindowMaxTiled = (int)(kBackSmem / (sizeof(float4) * kPairChunkMin));
+bool back_chunk_fits(int chunk, int window) { return (size_t)chunk * window * sizeof(float4) <= kBackSmem; }
+// the chunk asked for, or the largest one whose windows fit
+int back_chunk_for(int chunk, int window) {
+    if (chunk != 16 && chunk != 64) chunk = kPairChunk;
+    while (chunk > kPairChunkMin && !back_chunk_fits(chunk, window)) chunk /= 2;
+    return chunk;
+}
+size_t back_smem(int chunk, int window) {
+    return std::max((size_t)chunk * window * sizeof(float4), sizeof(float) * 2 * kPairRows * kPairThreads);
+}
+}  // namespace
+bool ctg_back_blocks_ok(const BackAngle *host_tab, int n_angles) {
+    for (int a = 0; a < n_angles; ++a)
+        if (!(fabsf(host_tab[a].cf) <= 1.0f && fabsf(host_tab[a].sf) <= 1.0f)) return false;
+    return true;
+}
+
+namespace {
+
+template <typename T, int kChunk>
+void launch_back_tiled(const T *b, ColRef bc, int N, int n_angles, int n_det, const BackAngle *tab,
+                       int window, const float *add, float *x, cudaStream_t st) {
+    const size_t smem = back_smem(kChunk, window);
+    const dim3 grid(back_tiles_x(N), back_tiles_y(N), kPairSplit);
+    pixel_back_tiled_kernel<T, kChunk><<<grid, kPairThreads, smem, st>>>(b, bc, N, n_angles, n_det, tab, window, add,
+                                                                      x);
+}
+
+// blocks: the 2 x 2 block kernel (ctg_back_blocks_ok).  back_chunk: angles
+// staged per pass (16, 32 or 64) of the one-pixel tiled kernel.  Each pixel sums
+// its angles in the same order whatever the chunk, so the result does not
+// depend on it.
+template <typename T>
+cudaError_t launch_back_t(const T *b, ColRef bc, int N, int n_angles, int n_det, const BackAngle *tab,
+                          int window, bool blocks, const float *add, float *x, cudaStream_t st, int back_chunk) {
+    if (blocks) {
+        const int nb = blk_nb(N);
+        const dim3 grid(back_tiles_x(N), blk_tiles_y(N, nb), kPairSplit);
+        if (nb == 4)
+            pixel_back_blocks_kernel<T, 4><<<grid, kBlkThreads, blk_smem(4), st>>>(b, bc, N, n_angles, n_det, tab, add, x);
+        else
+            pixel_back_blocks_kernel<T, 2><<<grid, kBlkThreads, blk_smem(2), st>>>(b, bc, N, n_angles, n_det, tab, add, x);
+    } else if (window > 0 && window <= kBackWindowMaxTiled) {
+        const int chunk = back_chunk_for(back_chunk, window);
+        if (chunk == 64) launch_back_tiled<T, 64>(b, bc, N, n_angles, n_det, tab, window, add, x, st);
+        else if (chunk == 16) launch_back_tiled<T, 16>(b, bc, N, n_angles, n_det, tab, window, add, x, st);
+        else if (chunk == 8) launch_back_tiled<T, 8>(b, bc, N, n_angles, n_det, tab, window, add, x, st);
+        else launch_back_tiled<T, kPairChunk>(b, bc, N, n_angles, n_det, tab, window, add, x, st);
+    } else {
+        dim3 grid((N + kBX - 1) / kBX, (N + kBY - 1) / kBY);
+        pixel_back_kernel<T><<<grid, dim3(kBX, kBY), 0, st>>>(b, bc, N, n_angles, n_det, tab, add, x);
+    }
+    return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_matched_tiled_t(const T *b, ColRef bc, int N, int n_angles, int n_det,
+                                   const BackAngle *tab, int window, const MatchedAngle *mt, float thr,
+                                   const float *add, float *x, cudaStream_t st) {
+    const int chunk = std::min(kPairChunk, back_chunk_for(kPairChunk, window));
+    const size_t smem = back_smem(chunk, window);
+    const dim3 grid(back_tiles_x(N), back_tiles_y(N), kPairSplit);
+    auto run = [&](auto kernel) {
+        kernel<<<grid, kPairThreads, smem, st>>>(b, bc, N, n_angles, n_det, tab, window, mt, thr, add, x);
+    };
+    if (chunk == kPairChunk) {
+        if (thr > 0.0f) run(matched_back_tiled_kernel<T, 2, kPairChunk>);
+        else run(matched_back_tiled_kernel<T, 1, kPairChunk>);
+    } else {
+        if (thr > 0.0f) run(matched_back_tiled_kernel<T, 2, 16>);
+        else run(matched_back_tiled_kernel<T, 1, 16>);
+    }
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t ctg_launch_back_matched_tiled(const void *b, int dtype, int N, int n_angles, int n_det,
+                                          const BackAngle *tab, int window, const MatchedAngle *mt,
+                                          float thr, const float *add, float *x, cudaStream_t st,
+                                          ColRef bc) {
+    if (window <= 0 || window > ctg_back_window_max()) return cudaErrorInvalidValue;
+    switch (dtype) {
+        case CTG_BASIS_FP32:
+            return launch_matched_tiled_t(static_cast<const float *>(b), bc, N, n_angles, n_det, tab, window,
+                                          mt, thr, add, x, st);
+        case CTG_BASIS_BF16:
+            return launch_matched_tiled_t(static_cast<const __nv_bfloat16 *>(b), bc, N, n_angles, n_det, tab,
+                                          window, mt, thr, add, x, st);
+        case CTG_BASIS_FP16:
+            return launch_matched_tiled_t(static_cast<const __half *>(b), bc, N, n_angles, n_det, tab, window,
+                                          mt, thr, add, x, st);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+cudaError_t ctg_launch_back(const void *b, int dtype, int N, int n_angles, int n_det,
+                            const BackAngle *tab, int window, bool blocks, const float *add, float *x,
+                            cudaStream_t st, int back_chunk, ColRef bc) {
+    switch (dtype) {
+        case CTG_BASIS_FP32:
+            return launch_back_t(static_cast<const float *>(b), bc, N, n_angles, n_det, tab, window, blocks, add, x,
+                                 st, back_chunk);
+        case CTG_BASIS_BF16:
+            return launch_back_t(static_cast<const __nv_bfloat16 *>(b), bc, N, n_angles, n_det, tab, window,
+                                 blocks, add, x, st, back_chunk);
+        case CTG_BASIS_FP16:
+            return launch_back_t(static_cast<const __half *>(b), bc, N, n_angles, n_det, tab, window, blocks, add,
+                                 x, st, back_chunk);
+        default: return cudaErrorInvalidValue;
+    }
+}

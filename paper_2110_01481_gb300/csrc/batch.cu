@@ -177,11 +177,8 @@ int upload_tables(InstPlan &p, cudaStream_t st) {
 // x = B b (+ add) with the instance's back projector
 cudaError_t back_inst(const InstPlan &p, const float *b, const float *add, float *x, cudaStream_t st) {
     const BatchInst &d = p.d;
-    if (d.back_model == CTG_BACK_PIXEL)
-        return ctg_launch_back(b, CTG_BASIS_FP32, p.g.N, p.g.n_angles, p.g.n_det, d.back, d.back_window,
-                               add, x, st);
-    return ctg_launch_back_matched_tiled(b, CTG_BASIS_FP32, p.g.N, p.g.n_angles, p.g.n_det, d.back,
-                                         d.back_window, d.mt, d.back_thr, add, x, st);
+    return ctg_batch_back_one(b, d.back_model, p.g.N, p.g.n_angles, p.g.n_det, d.back, d.back_window, d.mt,
+                              d.back_thr, add, x, st);
 }
 
 RedScratch scratch_of(const BatchInst &d) {

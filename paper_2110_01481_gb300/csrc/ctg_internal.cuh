@@ -92,7 +92,7 @@ __device__ __forceinline__ size_t col_offset(const ColRef &c) {
 }
 #endif
 
-// ---- projector launchers (projectors.cu) --------------------------------
+// ---- projector launchers (projectors.cu, back.cu) --------------------------------
 // Stage x (n elements of type `dtype`, a CTG_BASIS_* value; column xc of a
 // basis at x when xc.k is set) for the forward projector.
 cudaError_t ctg_launch_pad(const void *x, int dtype, float2 *pad, int N, const PadLayout &pl,
@@ -144,13 +144,17 @@ bool ctg_forward_split_safe(const FwdAngle *host_tab, int N, int n_angles, int n
 // Detector-window width (in bins) that the tiled back projector stages per
 // angle, from the host copy of the angle table.
 int ctg_back_window(const BackAngle *host_tab, int n_angles);
+// Whether the pixel-driven B may take 2 x 2 pixel blocks: no angle moves more
+// than one detector bin per pixel step (every pitch of a pixel or more).
+bool ctg_back_blocks_ok(const BackAngle *host_tab, int n_angles);
 // x = B b (+ add, if add != NULL); b has element type `dtype`; window from
 // ctg_back_window
+// blocks: ctg_back_blocks_ok's answer for the table.
 // back_chunk: angles staged per pass, 16, 32 or 64 (tuned like the forward shape;
-// the result does not depend on it).
+// the result does not depend on it, and the block kernel does not use it).
 // bc: the input is column bc of a basis at b (bc.k set), or b itself.
 cudaError_t ctg_launch_back(const void *b, int dtype, int N, int n_angles, int n_det,
-                            const BackAngle *tab, int window, const float *add, float *x,
+                            const BackAngle *tab, int window, bool blocks, const float *add, float *x,
                             cudaStream_t st, int back_chunk = 32, ColRef bc = col_none());
 
 // ---- matched back projector (matched.cu) ----------------------------------
@@ -160,7 +164,7 @@ cudaError_t ctg_launch_back(const void *b, int dtype, int N, int n_angles, int n
 cudaError_t ctg_launch_back_matched(const void *b, int dtype, int N, int n_angles, int n_det,
                                     const BackAngle *tab, const MatchedAngle *mt, int rm, float thr,
                                     const float *add, float *x, cudaStream_t st, ColRef bc = col_none());
-// The same with the tiled design of the pixel-driven B (projectors.cu), for
+// The same with the tiled design of the pixel-driven B (back.cu), for
 // rm = 0 and window <= ctg_back_window_max().
 cudaError_t ctg_launch_back_matched_tiled(const void *b, int dtype, int N, int n_angles, int n_det,
                                           const BackAngle *tab, int window, const MatchedAngle *mt,
@@ -425,6 +429,11 @@ struct BatchInst {
 // otherwise 32); the result does not depend on it.
 cudaError_t ctg_batch_back(BatchInst *insts, const int2 *map, int nblocks, int max_window,
                            cudaStream_t st, int wtype = CTG_BASIS_FP32, int chunk = 32);
+// x = B b (+ add) of one solve of a batch (back_model, weights mt, threshold
+// thr), by the tile of ctg_batch_back.
+cudaError_t ctg_batch_back_one(const float *b, int back_model, int N, int n_angles, int n_det,
+                               const BackAngle *tab, int window, const MatchedAngle *mt, float thr,
+                               const float *add, float *x, cudaStream_t st);
 bool ctg_batch_back_chunk_ok(int chunk, int max_window);
 // Staging for the forward projector: AB stages t = B w_k (variant CTG_AB);
 // BA stages w_{k+1}, with x_k interleaved when it has the DP stop

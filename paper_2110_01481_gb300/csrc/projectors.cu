@@ -1,20 +1,19 @@
 // Matrix-free projectors of the unmatched pair (A, B) (paper Sec. 1,
 // eq. (1.1)-(1.2)): the Joseph ray-driven forward projector A, one thread
-// per ray, and the pixel-driven back projector B, one thread per pixel
-// (four pixels per thread), gather-only (no atomics).
+// per ray, and the back projector of batched and served solves, one thread
+// per pixel (four pixels per thread), gather-only (no atomics).  The single
+// launches' back projectors are in back.cu.
 //
 // Both kernels read their input as (value, forward difference) pairs, so one
 // 8-byte load and one FMA give a linear interpolation:
 //   lerp(v, j + f) = v[j] + f (v[j+1] - v[j]).
 #include <cooperative_groups.h>
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
 
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
 
-#include "ctg_internal.cuh"
+#include "proj_device.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -22,11 +21,6 @@ namespace {
 
 constexpr int kPadTile = 32;
 constexpr int kPadRows = 8;    // staging blocks are kPadTile x kPadRows threads
-
-// Inputs that are Krylov basis vectors may be stored in BF16 or FP16.
-__device__ __forceinline__ float to_f(float v) { return v; }
-__device__ __forceinline__ float to_f(__nv_bfloat16 v) { return __bfloat162float(v); }
-__device__ __forceinline__ float to_f(__half v) { return __half2float(v); }
 
 __device__ __forceinline__ float2 lerp_pair(float v0, float v1) {
     // (v0 - dv, dv): with m = 1 + f, (v0 - dv) + m dv = v0 + f dv
@@ -124,30 +118,6 @@ template <int kImgs, typename T>
 __global__ void pad_pairs_kernel(const T *__restrict__ x, ColRef xc, const float *__restrict__ x2,
                                  void *__restrict__ pad, int N, int stride, int border) {
     pad_pairs_block<kImgs, T>(x + col_offset(xc), x2, pad, N, stride, border, blockIdx.x, blockIdx.y);
-}
-
-__device__ __forceinline__ float fx_frac(long long U) {
-    // top 24 bits of the 40-bit fraction of a 24.40 value, in [0, 1)
-    const unsigned f24 = (unsigned)((unsigned long long)U >> (CTG_FX_BITS - 24)) & 0xFFFFFFu;
-    return (float)f24 * (1.0f / 16777216.0f);
-}
-
-// floor(u) by the round-down magic-number add, for two positions at once in
-// packed FP32 pairs: t = u + M rounded down (M = 1.5 * 2^23, so the low
-// mantissa bits of t hold floor(u) for 0 <= u < 2^22) and f = u - (t - M),
-// exactly the scalar sequence per position, with half the instructions.
-__device__ __forceinline__ void floor_frac2(float u0, float u1, float &t0, float &t1, float &f0,
-                                            float &f1) {
-    asm("{\n\t.reg .b64 u, m, t, f;\n\t"
-        "mov.b64 u, {%4, %5};\n\t"
-        "mov.b64 m, {%6, %6};\n\t"
-        "add.rm.f32x2 t, u, m;\n\t"
-        "sub.rn.f32x2 f, t, m;\n\t"
-        "sub.rn.f32x2 f, u, f;\n\t"
-        "mov.b64 {%0, %1}, t;\n\t"
-        "mov.b64 {%2, %3}, f;\n\t}"
-        : "=f"(t0), "=f"(t1), "=f"(f0), "=f"(f1)
-        : "f"(u0), "f"(u1), "f"(12582912.0f));
 }
 
 __device__ __forceinline__ float one_plus_frac(unsigned lo) {
@@ -291,7 +261,13 @@ joseph_forward_kernel(const void *__restrict__ pad, int N, int stride, int borde
 }
 
 // ---------------------------------------------------------------------------
-// Pixel-driven back projection.  A thread-block cluster of kBSplit CTAs owns
+// Back projection of batched and served solves.  (Single launches have faster
+// kernels, back.cu.  Their positions and sums round differently, about 1e-7
+// of B b; a solve of a batch may run to steps where the iterate is an
+// ill-conditioned function of the rounding and moves by 1e-3, so batches keep
+// this kernel's sums: measured with the 2 x 2 block kernel in its place,
+// iterates at k >= 20 moved by up to 5e-3 for 10 % of the time.)
+// A thread-block cluster of kBSplit CTAs owns
 // a 32 x 32 pixel tile; each CTA (256 threads, four rows each) sums a
 // contiguous quarter of the angles.  For a chunk of angles a CTA stages, per
 // angle, the detector window that the tile projects onto as
@@ -305,8 +281,6 @@ joseph_forward_kernel(const void *__restrict__ pad, int N, int stride, int borde
 constexpr int kBT = 32;          // tile side
 constexpr int kBRows = 4;        // rows per thread (threads: 32 x 8), batched launches
 constexpr int kBThreads = 256;
-constexpr int kBRowsTiled = 4;   // rows per thread of the single launch (8 rows and 32 x 4
-                                 // threads measured 6 % slower: fewer warps to hide latency)
 template <int kRows>
 __host__ __device__ constexpr int back_threads() { return kBT * (kBT / kRows); }
 constexpr int kBChunk = 32;      // angles staged per pass
@@ -435,70 +409,13 @@ __device__ __forceinline__ void pixel_back_tile(const T *__restrict__ b, int N, 
     cluster.sync();   // peers' shared memory must outlive the reads above
 }
 
-// bc: the input is column bc of a basis (b + col_offset(bc)), or b itself.
-template <typename T, int kChunk>
-__global__ void __cluster_dims__(1, 1, kBSplit) __launch_bounds__(back_threads<kBRowsTiled>())
-pixel_back_tiled_kernel(const T *__restrict__ b, ColRef bc, int N, int n_angles, int n_det,
-                        const BackAngle *__restrict__ tab, int W, const float *__restrict__ add,
-                        float *__restrict__ x) {
-    pixel_back_tile<T, 0, kChunk, kBRowsTiled>(b + col_offset(bc), N, n_angles, n_det, tab, W, add, x,
-                                               blockIdx.x, blockIdx.y);
-}
-
-// A^T (kModel 1) or B_tau (kModel 2) with the tiled design above.
-template <typename T, int kModel>
+// One solve of a batch on its own (its start and exit): the same tile.
+template <int kModel>
 __global__ void __cluster_dims__(1, 1, kBSplit) __launch_bounds__(kBThreads)
-matched_back_tiled_kernel(const T *__restrict__ b, ColRef bc, int N, int n_angles, int n_det,
-                          const BackAngle *__restrict__ tab, int W, const MatchedAngle *__restrict__ mt,
-                          float thr, const float *__restrict__ add, float *__restrict__ x) {
-    pixel_back_tile<T, kModel>(b + col_offset(bc), N, n_angles, n_det, tab, W, add, x, blockIdx.x, blockIdx.y,
-                               mt, thr);
-}
-
-// Generic pixel-driven back projection (any detector pitch): 32 x 8 tiles,
-// taps read through L1 with bounds tests.
-constexpr int kBX = 32, kBY = 8, kAChunk = 256;
-
-template <typename T>
-__global__ void __launch_bounds__(kBX *kBY)
-pixel_back_kernel(const T *__restrict__ b, ColRef bc, int N, int n_angles, int n_det,
-                  const BackAngle *__restrict__ tab, const float *__restrict__ add,
-                  float *__restrict__ x) {
-    __shared__ float4 sp[kAChunk];
-    b += col_offset(bc);
-    const int j0 = blockIdx.x * kBX, i0 = blockIdx.y * kBY;
-    const int dj = threadIdx.x, di = threadIdx.y;
-    const int tid = di * kBX + dj;
-    const float fdj = (float)dj, fdi = (float)di;
-    float acc = 0.0f;
-    for (int a0 = 0; a0 < n_angles; a0 += kAChunk) {
-        const int na = min(kAChunk, n_angles - a0);
-        __syncthreads();
-        if (tid < na) {
-            const BackAngle t = tab[a0 + tid];
-            const long long U0 = t.C + (long long)j0 * t.COS + (long long)i0 * t.SIN;
-            sp[tid] = make_float4(t.cf, t.sf, fx_frac(U0),
-                                  __int_as_float((int)(U0 >> CTG_FX_BITS)));
-        }
-        __syncthreads();
-        const T *brow = b + (size_t)a0 * n_det;
-#pragma unroll 4
-        for (int k = 0; k < na; ++k, brow += n_det) {
-            const float4 p = sp[k];
-            const float u = fmaf(fdi, p.y, fmaf(fdj, p.x, p.z));
-            const float fl = floorf(u);
-            const int dd = __float_as_int(p.w) + (int)fl;
-            const float f = u - fl;
-            const float v0 = ((unsigned)dd < (unsigned)n_det) ? to_f(__ldg(brow + dd)) : 0.0f;
-            const float v1 = ((unsigned)(dd + 1) < (unsigned)n_det) ? to_f(__ldg(brow + dd + 1)) : 0.0f;
-            acc += fmaf(f, v1 - v0, v0);
-        }
-    }
-    const int i = i0 + di, j = j0 + dj;
-    if (i < N && j < N) {
-        const size_t p = (size_t)i * N + j;
-        x[p] = add ? acc + add[p] : acc;
-    }
+batch_back_one_kernel(const float *__restrict__ b, int N, int n_angles, int n_det,
+                      const BackAngle *__restrict__ tab, int W, const MatchedAngle *__restrict__ mt, float thr,
+                      const float *__restrict__ add, float *__restrict__ x) {
+    pixel_back_tile<float, kModel>(b, N, n_angles, n_det, tab, W, add, x, blockIdx.x, blockIdx.y, mt, thr);
 }
 
 // ---- batched kernels: one launch for the same phase of every instance ----
@@ -628,6 +545,21 @@ void batch_back_t(BatchInst *insts, const int2 *map, int nblocks, int max_window
         batch_back_kernel<float, kChunk><<<grid, kBThreads, smem, st>>>(insts, map);
 }
 }  // namespace
+
+cudaError_t ctg_batch_back_one(const float *b, int back_model, int N, int n_angles, int n_det,
+                               const BackAngle *tab, int window, const MatchedAngle *mt, float thr,
+                               const float *add, float *x, cudaStream_t st) {
+    if (window <= 0 || window > ctg_back_window_max()) return cudaErrorInvalidValue;
+    const size_t smem = sizeof(float2) * (size_t)kBChunk * window;
+    const dim3 grid((N + kBT - 1) / kBT, (N + kBT - 1) / kBT, kBSplit);
+    auto run = [&](auto kernel) {
+        kernel<<<grid, kBThreads, smem, st>>>(b, N, n_angles, n_det, tab, window, mt, thr, add, x);
+    };
+    if (back_model == CTG_BACK_PIXEL) run(batch_back_one_kernel<0>);
+    else if (thr > 0.0f) run(batch_back_one_kernel<2>);
+    else run(batch_back_one_kernel<1>);
+    return cudaGetLastError();
+}
 
 bool ctg_batch_back_chunk_ok(int chunk, int max_window) {
     return (chunk == 16 || chunk == 32 || chunk == 64) && (size_t)chunk * max_window * sizeof(float2) <= 40 * 1024;
@@ -858,88 +790,4 @@ bool ctg_forward_split_safe(const FwdAngle *tab, int N, int n_angles, int n_det,
             }
         }
     return true;
-}
-
-namespace {
-
-template <typename T, int kChunk>
-void launch_back_tiled(const T *b, ColRef bc, int N, int n_angles, int n_det, const BackAngle *tab,
-                       int window, const float *add, float *x, cudaStream_t st) {
-    const size_t smem = sizeof(float2) * (size_t)kChunk * window;
-    const dim3 grid((N + kBT - 1) / kBT, (N + kBT - 1) / kBT, kBSplit);
-    pixel_back_tiled_kernel<T, kChunk><<<grid, back_threads<kBRowsTiled>(), smem, st>>>(b, bc, N, n_angles, n_det, tab,
-                                                                      window, add, x);
-}
-
-// back_chunk: angles staged per pass (16, 32 or 64).  Each pixel sums its
-// angles in the same order whatever the chunk, so the result does not
-// depend on it.
-template <typename T>
-cudaError_t launch_back_t(const T *b, ColRef bc, int N, int n_angles, int n_det, const BackAngle *tab,
-                          int window, const float *add, float *x, cudaStream_t st, int back_chunk) {
-    const size_t bytes_per_angle = sizeof(float2) * (size_t)window;
-    if (window > 0 && back_chunk == 64 && 64 * bytes_per_angle <= 40 * 1024) {
-        launch_back_tiled<T, 64>(b, bc, N, n_angles, n_det, tab, window, add, x, st);
-    } else if (window > 0 && back_chunk == 16 && 16 * bytes_per_angle <= 40 * 1024) {
-        launch_back_tiled<T, 16>(b, bc, N, n_angles, n_det, tab, window, add, x, st);
-    } else if (window > 0 && kBChunk * bytes_per_angle <= 40 * 1024) {
-        launch_back_tiled<T, kBChunk>(b, bc, N, n_angles, n_det, tab, window, add, x, st);
-    } else {
-        dim3 grid((N + kBX - 1) / kBX, (N + kBY - 1) / kBY);
-        pixel_back_kernel<T><<<grid, dim3(kBX, kBY), 0, st>>>(b, bc, N, n_angles, n_det, tab, add, x);
-    }
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_matched_tiled_t(const T *b, ColRef bc, int N, int n_angles, int n_det,
-                                   const BackAngle *tab, int window, const MatchedAngle *mt, float thr,
-                                   const float *add, float *x, cudaStream_t st) {
-    const size_t smem = sizeof(float2) * (size_t)kBChunk * window;
-    const dim3 grid((N + kBT - 1) / kBT, (N + kBT - 1) / kBT, kBSplit);
-    if (thr > 0.0f)
-        matched_back_tiled_kernel<T, 2><<<grid, kBThreads, smem, st>>>(b, bc, N, n_angles, n_det, tab,
-                                                                       window, mt, thr, add, x);
-    else
-        matched_back_tiled_kernel<T, 1><<<grid, kBThreads, smem, st>>>(b, bc, N, n_angles, n_det, tab,
-                                                                       window, mt, thr, add, x);
-    return cudaGetLastError();
-}
-
-}  // namespace
-
-cudaError_t ctg_launch_back_matched_tiled(const void *b, int dtype, int N, int n_angles, int n_det,
-                                          const BackAngle *tab, int window, const MatchedAngle *mt,
-                                          float thr, const float *add, float *x, cudaStream_t st,
-                                          ColRef bc) {
-    if (window <= 0 || window > ctg_back_window_max()) return cudaErrorInvalidValue;
-    switch (dtype) {
-        case CTG_BASIS_FP32:
-            return launch_matched_tiled_t(static_cast<const float *>(b), bc, N, n_angles, n_det, tab, window,
-                                          mt, thr, add, x, st);
-        case CTG_BASIS_BF16:
-            return launch_matched_tiled_t(static_cast<const __nv_bfloat16 *>(b), bc, N, n_angles, n_det, tab,
-                                          window, mt, thr, add, x, st);
-        case CTG_BASIS_FP16:
-            return launch_matched_tiled_t(static_cast<const __half *>(b), bc, N, n_angles, n_det, tab, window,
-                                          mt, thr, add, x, st);
-        default: return cudaErrorInvalidValue;
-    }
-}
-
-cudaError_t ctg_launch_back(const void *b, int dtype, int N, int n_angles, int n_det,
-                            const BackAngle *tab, int window, const float *add, float *x,
-                            cudaStream_t st, int back_chunk, ColRef bc) {
-    switch (dtype) {
-        case CTG_BASIS_FP32:
-            return launch_back_t(static_cast<const float *>(b), bc, N, n_angles, n_det, tab, window, add, x, st,
-                                 back_chunk);
-        case CTG_BASIS_BF16:
-            return launch_back_t(static_cast<const __nv_bfloat16 *>(b), bc, N, n_angles, n_det, tab, window,
-                                 add, x, st, back_chunk);
-        case CTG_BASIS_FP16:
-            return launch_back_t(static_cast<const __half *>(b), bc, N, n_angles, n_det, tab, window, add, x,
-                                 st, back_chunk);
-        default: return cudaErrorInvalidValue;
-    }
 }
