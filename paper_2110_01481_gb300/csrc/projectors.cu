@@ -176,6 +176,10 @@ __device__ __forceinline__ void joseph_forward_block(const void *__restrict__ pa
             const float tlo = fmaxf(fminf(r1, r2), -2.0f), thi = fminf(fmaxf(r1, r2), (float)N + 1);
             lo = max(0, (int)floorf(tlo) - 1);
             hi = min(N - 1, (int)ceilf(thi) + 1);
+            // a ray that misses the image: the empty range of every other
+            // such lane, so that it does not widen the warp's walk (rounded
+            // down to a multiple of 4, it could start one far from the image)
+            if (lo > hi) lo = N, hi = -1;
         } else if (u0 > -2.0f && u0 < (float)N + 1.0f) {
             lo = 0;
             hi = N - 1;
@@ -682,36 +686,50 @@ void launch_forward_shape(int shape, const void *pad, int N, const PadLayout &pl
 }
 
 // walk range [lo, hi] of ray d of angle t, as joseph_forward_block
-// estimates it (host arithmetic; may differ from the device's by a step)
-void ray_range(const FwdAngle &t, int N, int d, int &lo, int &hi) {
+// estimates it (host arithmetic; may differ from the device's by a step).
+// Returns 0 for a ray that meets the image; for one that misses it (lo = N, hi
+// = -1), -1 or 1 as its crossing lies before the first or past the last row.
+int ray_range(const FwdAngle &t, int N, int d, int &lo, int &hi) {
     const float u0 = (float)d * t.pf + t.qf;
     lo = N;
     hi = -1;
     if (std::fabs(t.df) > 1e-20f) {
         const float r1 = (-1.0f - u0) / t.df, r2 = ((float)N - u0) / t.df;
-        const float tlo = std::max(std::min(r1, r2), -2.0f);
-        const float thi = std::min(std::max(r1, r2), (float)N + 1);
-        lo = std::max(0, (int)std::floor(tlo) - 1);
-        hi = std::min(N - 1, (int)std::ceil(thi) + 1);
-    } else if (u0 > -2.0f && u0 < (float)N + 1.0f) {
+        const float tlo = std::max(std::min(r1, r2), -2.0f), thi = std::min(std::max(r1, r2), (float)N + 1);
+        const float flo = std::floor(tlo) - 1.0f, fhi = std::ceil(thi) + 1.0f;
+        if (fhi < 0.0f) return -1;
+        if (flo > (float)(N - 1)) return 1;
+        lo = std::max(0, (int)flo);
+        hi = std::min(N - 1, (int)fhi);
+        if (lo <= hi) return 0;
+        lo = N;
+        hi = -1;
+        return 1;
+    }
+    if (u0 > -2.0f && u0 < (float)N + 1.0f) {
         lo = 0;
         hi = N - 1;
+        return 0;
     }
+    return u0 < 0.0f ? -1 : 1;
 }
 
 // union walk range of rays d0 .. d1 - 1 of angle t: a ray's range ends are
-// clamped linear functions of d, so the first and last ray give it (all
-// rays when the walk is parallel to the detector, D = 0)
+// clamped linear functions of d, so where the first and the last ray meet the
+// image they give it, and where both miss it on the same side so do all others
+// (else, and for a walk parallel to the detector, D = 0, all rays are asked)
 void group_range(const FwdAngle &t, int N, int d0, int d1, int &wlo, int &whi) {
-    const bool all = !(std::fabs(t.df) > 1e-20f);
-    wlo = N;
-    whi = -1;
-    for (int d = d0; d < d1; d += (all || d + 1 == d1) ? 1 : d1 - 1 - d) {
-        int lo, hi;
-        ray_range(t, N, d, lo, hi);
-        wlo = std::min(wlo, lo);
-        whi = std::max(whi, hi);
-    }
+    int lo, hi;
+    const int first = ray_range(t, N, d0, wlo, whi), last = ray_range(t, N, d1 - 1, lo, hi);
+    const bool all = !(std::fabs(t.df) > 1e-20f) || first != last;
+    wlo = std::min(wlo, lo);
+    whi = std::max(whi, hi);
+    if (all)
+        for (int d = d0 + 1; d < d1 - 1; ++d) {
+            ray_range(t, N, d, lo, hi);
+            wlo = std::min(wlo, lo);
+            whi = std::max(whi, hi);
+        }
 }
 
 }  // namespace
