@@ -32,18 +32,14 @@ namespace {
 // memory in rank order (deterministic, no atomics), each CTA finishing a share
 // of the tile's rows.
 // Bound by the shared-memory data path (8 bytes per interpolation, 16 per clock
-// and SM; 2048^2, 1800 angles run at 80 % of that): the pixel-driven B at 512^2,
-// 720 angles takes 63 us and at 2048^2 1,908 us, against 73 and 2,381 us with one
-// pixel per position.
+// and SM; the pixel-driven B at 2048^2, 1800 angles runs at 80 % of that); with
+// one pixel per position it was bound by issue slots.  A^T at 512^2, 720 angles
+// 103 -> 70 us, at 1001^2, 900 angles 466 -> 280 us.
 constexpr int kPT = 32;             // tile side
-constexpr int kPairRows = 8;        // rows per thread (threads: 32 x 4): the shared parameter load and the
-                                    // address base of an angle serve 16 interpolations (512^2, 720 angles:
-                                    // 63 us against 67 with 4 rows and 256 threads)
-constexpr int kPairThreads = 128;
 template <int kRows>
 __host__ __device__ constexpr int pair_threads() { return kPT * (kPT / kRows); }
 constexpr int kPairChunk = 32;      // angles staged per pass
-constexpr int kPairSplit = 8;       // CTAs per cluster = angle groups per tile (512^2: 63 us, 76 us with 4)
+constexpr int kMaxSplit = 8;        // CTAs per cluster = angle groups per tile, at most (portable clusters)
 // tiles of an image: columns x rows of the upper half
 __host__ __device__ constexpr int back_tiles_x(int N) { return (N + kPT - 1) / kPT; }
 __host__ __device__ constexpr int back_tiles_y(int N) { return ((N + 1) / 2 + kPT - 1) / kPT; }
@@ -68,7 +64,7 @@ __device__ __forceinline__ void add2(float &a0, float &a1, float v0, float v1) {
 // for the pixel-driven B and (b[d], b'[d], b[d+1], b'[d+1]) for the others.
 // kRows: pixel rows per thread, kPT / kRows row threads per column (rows
 // di, di + kPT / kRows, ...).
-template <typename T, int kModel = 0, int kChunk = kPairChunk, int kRows = kPairRows, int kSplit = kPairSplit>
+template <typename T, int kModel, int kChunk, int kRows, int kSplit>
 __device__ __forceinline__ void pixel_pair_tile(const T *__restrict__ b, int N, int n_angles,
                                                 int n_det, const BackAngle *__restrict__ tab,
                                                 int W, const float *__restrict__ add,
@@ -90,9 +86,9 @@ __device__ __forceinline__ void pixel_pair_tile(const T *__restrict__ b, int N, 
     const int per = (n_angles + kSplit - 1) / kSplit;
     const int a_begin = min(n_angles, rank * per), a_end = min(n_angles, a_begin + per);
     const int wc = W / 2;                             // window entry of the tile centre's bin
-    float acc[kRows][2];                              // direct and reflected pixel
+    float sum[kRows][2], acc[kRows][2];               // direct and reflected pixel; of the latest 32 angles
 #pragma unroll
-    for (int r = 0; r < kRows; ++r) acc[r][0] = acc[r][1] = 0.f;
+    for (int r = 0; r < kRows; ++r) sum[r][0] = sum[r][1] = acc[r][0] = acc[r][1] = 0.f;
     for (int a0 = a_begin; a0 < a_end; a0 += kChunk) {
         const int na = min(kChunk, a_end - a0);
         __syncthreads();
@@ -160,12 +156,20 @@ __device__ __forceinline__ void pixel_pair_tile(const T *__restrict__ b, int N, 
                 }
             }
         }
+        // 32 angles at a time (whatever the chunk), which keeps the chains of
+        // additions short for every split
+        if ((a0 - a_begin + kChunk) % kPairChunk == 0 || a0 + kChunk >= a_end)
+#pragma unroll
+            for (int r = 0; r < kRows; ++r) {
+                add2(sum[r][0], sum[r][1], acc[r][0], acc[r][1]);
+                acc[r][0] = acc[r][1] = 0.f;
+            }
     }
     __syncthreads();                                  // the windows have been read
 #pragma unroll
     for (int r = 0; r < kRows; ++r) {
-        s_part[(2 * r) * kThr + threadIdx.x] = acc[r][0];
-        s_part[(2 * r + 1) * kThr + threadIdx.x] = acc[r][1];
+        s_part[(2 * r) * kThr + threadIdx.x] = sum[r][0];
+        s_part[(2 * r + 1) * kThr + threadIdx.x] = sum[r][1];
     }
     cluster.sync();
     // this CTA finishes planes rank, rank + kSplit, ...: plane 2 r + h holds
@@ -175,14 +179,14 @@ __device__ __forceinline__ void pixel_pair_tile(const T *__restrict__ b, int N, 
     const long long last = (long long)N * N - 1;
 #pragma unroll
     for (int q = rank; q < 2 * kRows; q += kSplit) {
-        float sum = 0.0f;
+        float all = 0.0f;
 #pragma unroll
-        for (int c = 0; c < kSplit; ++c) sum += cluster.map_shared_rank(s_part + q * kThr, c)[threadIdx.x];
+        for (int c = 0; c < kSplit; ++c) all += cluster.map_shared_rank(s_part + q * kThr, c)[threadIdx.x];
         const int i = i0 + di + kRT * (q >> 1), j = j0 + dj;
         const long long p = (long long)i * N + j;
         if (i < N && j < N && ((q & 1) ? 2 * p < last : 2 * p <= last)) {
             const long long o = (q & 1) ? last - p : p;
-            x[o] = add ? sum + add[o] : sum;
+            x[o] = add ? all + add[o] : all;
         }
     }
     cluster.sync();   // peers' shared memory must outlive the reads above
@@ -215,7 +219,7 @@ __device__ __forceinline__ void pixel_pair_tile(const T *__restrict__ b, int N, 
 // interpolations/s), 2048^2, 1800 angles 2,381 -> 1,399 us (5.4 T/s).
 constexpr int kBlkWarps = 4, kBlkThreads = 32 * kBlkWarps;
 constexpr int kBlkChunk = 16;         // angles per stage, two stages in flight
-constexpr int kBlkFlush = 4;
+constexpr int kBlkFlush = 4;          // (1 in the smaller clusters: few angles, so few chains to average over)
 // Window of a 32 x th tile: a block's lowest corner lies within half the tile's
 // diagonal of the centre (21.92 bins for 32 rows, 35.11 for 64) plus a phase below
 // one, and reads the three bins after its own.
@@ -276,13 +280,14 @@ __device__ __noinline__ void pixel_back_plain(const T *__restrict__ b, int n_det
 // Body of one CTA of the cluster for the 32 x (16 kNB) tile (bx, by) of the
 // upper half; each of the 128 threads owns kNB blocks 16 rows apart.  Every CTA
 // of a cluster must call it.
-template <typename T, int kNB, int kSplit = kPairSplit>
+template <typename T, int kNB, int kSplit>
 __device__ __forceinline__ void pixel_back_blocks(const T *__restrict__ b, int N, int n_angles, int n_det,
                                                   const BackAngle *__restrict__ tab,
                                                   const float *__restrict__ add, float *__restrict__ x, int bx,
                                                   int by) {
     constexpr int kThr = kBlkThreads, kStep = 4 * kBlkWarps, kTH = kStep * kNB;   // rows between blocks; tile height
     constexpr int kWin = blk_window(kTH), kCentre = blk_centre(kTH);
+    constexpr int kFlush = kSplit == kMaxSplit ? kBlkFlush : 1;
     extern __shared__ float4 s_dyn[];
     float2 *s_win = reinterpret_cast<float2 *>(s_dyn);            // [2][kBlkChunk][kWin] (b, b')
     float *s_px = reinterpret_cast<float *>(s_win + 2 * kBlkChunk * kWin);   // [2][kTH][32] sums of the pixels
@@ -442,7 +447,7 @@ __device__ __forceinline__ void pixel_back_blocks(const T *__restrict__ b, int N
                 }
             }
         }
-        if (c % kBlkFlush == kBlkFlush - 1) flush(right);
+        if (c % kFlush == kFlush - 1) flush(right);
     }
     flush(right);
     {
@@ -480,37 +485,24 @@ __device__ __forceinline__ void pixel_back_blocks(const T *__restrict__ b, int N
 constexpr size_t blk_smem(int nb) {
     return sizeof(float2) * 2 * kBlkChunk * blk_window(16 * nb) + sizeof(float) * 2 * 16 * nb * kPT;
 }
-// Blocks per thread for an image: four (64-row tiles, half the staging and
-// parameter loads per pixel) once that leaves about three CTAs per SM, else two
-// (512^2: 49 against 51.5 us, 2048^2: 1,399 against 1,489; 361^2: 14.2 against 12.5).
 constexpr int blk_tiles_y(int N, int nb) { return ((N + 1) / 2 + 16 * nb - 1) / (16 * nb); }
-constexpr int blk_nb(int N) { return back_tiles_x(N) * blk_tiles_y(N, 4) * kPairSplit >= 456 ? 4 : 2; }
 
-template <typename T, int kNB>
-__global__ void __cluster_dims__(1, 1, kPairSplit) __launch_bounds__(kBlkThreads, kNB == 4 ? 4 : 7)
+template <typename T, int kNB, int kSplit>
+__global__ void __cluster_dims__(1, 1, kSplit) __launch_bounds__(kBlkThreads, kNB == 4 ? 4 : 7)
 pixel_back_blocks_kernel(const T *__restrict__ b, ColRef bc, int N, int n_angles, int n_det,
                          const BackAngle *__restrict__ tab, const float *__restrict__ add, float *__restrict__ x) {
-    pixel_back_blocks<T, kNB>(b + col_offset(bc), N, n_angles, n_det, tab, add, x, blockIdx.x, blockIdx.y);
+    pixel_back_blocks<T, kNB, kSplit>(b + col_offset(bc), N, n_angles, n_det, tab, add, x, blockIdx.x, blockIdx.y);
 }
 
 // bc: the input is column bc of a basis (b + col_offset(bc)), or b itself.
-template <typename T, int kChunk>
-__global__ void __cluster_dims__(1, 1, kPairSplit) __launch_bounds__(kPairThreads)
-pixel_back_tiled_kernel(const T *__restrict__ b, ColRef bc, int N, int n_angles, int n_det,
-                        const BackAngle *__restrict__ tab, int W, const float *__restrict__ add,
-                        float *__restrict__ x) {
-    pixel_pair_tile<T, 0, kChunk, kPairRows>(b + col_offset(bc), N, n_angles, n_det, tab, W, add, x,
-                                               blockIdx.x, blockIdx.y);
-}
-
-// A^T (kModel 1) or B_tau (kModel 2) with the tiled design above.
-template <typename T, int kModel, int kChunk>
-__global__ void __cluster_dims__(1, 1, kPairSplit) __launch_bounds__(kPairThreads)
-matched_back_tiled_kernel(const T *__restrict__ b, ColRef bc, int N, int n_angles, int n_det,
-                          const BackAngle *__restrict__ tab, int W, const MatchedAngle *__restrict__ mt,
-                          float thr, const float *__restrict__ add, float *__restrict__ x) {
-    pixel_pair_tile<T, kModel, kChunk>(b + col_offset(bc), N, n_angles, n_det, tab, W, add, x, blockIdx.x, blockIdx.y,
-                               mt, thr);
+// kModel: the pixel-driven B (0), A^T (1) or B_tau (2).
+template <typename T, int kModel, int kChunk, int kRows, int kSplit>
+__global__ void __cluster_dims__(1, 1, kSplit) __launch_bounds__(pair_threads<kRows>())
+pixel_pair_kernel(const T *__restrict__ b, ColRef bc, int N, int n_angles, int n_det,
+                  const BackAngle *__restrict__ tab, int W, const MatchedAngle *__restrict__ mt, float thr,
+                  const float *__restrict__ add, float *__restrict__ x) {
+    pixel_pair_tile<T, kModel, kChunk, kRows, kSplit>(b + col_offset(bc), N, n_angles, n_det, tab, W, add, x,
+                                                      blockIdx.x, blockIdx.y, mt, thr);
 }
 
 // Generic pixel-driven back projection (any detector pitch): 32 x 8 tiles,
@@ -571,14 +563,35 @@ constexpr int kBackWindowMaxTiled = (int)(kBackSmem / (sizeof(float4) * kPairChu
 bool back_chunk_fits(int chunk, int window) { return (size_t)chunk * window * sizeof(float4) <= kBackSmem; }
 // the chunk asked for, or the largest one whose windows fit
 int back_chunk_for(int chunk, int window) {
-    if (chunk != 16 && chunk != 64) chunk = kPairChunk;
+    if (chunk != 16) chunk = kPairChunk;
     while (chunk > kPairChunkMin && !back_chunk_fits(chunk, window)) chunk /= 2;
     return chunk;
 }
-size_t back_smem(int chunk, int window) {
-    return std::max((size_t)chunk * window * sizeof(float4), sizeof(float) * 2 * kPairRows * kPairThreads);
+size_t pair_smem(int chunk, int window) {
+    return std::max((size_t)chunk * window * sizeof(float4), sizeof(float) * 2 * kPT * kPT);
+}
+
+// CTAs per cluster for an image of `tiles` tiles: eight, halved while a CTA's
+// share would be below 30 angles (a tile's start, end and cluster sum then cost
+// as much as its angles) and the launch keeps about three CTAs per SM.  B at
+// 1024^2: 60 angles 31 us with 8, 21 with 2; 120 angles 39 and 35 (4); 2048^2, 60
+// angles 104 and 66 us.
+constexpr int kFullGrid = 450;
+int split_for(int n_angles, int tiles) {
+    int s = kMaxSplit;
+    while (s > 2 && n_angles < 30 * s && tiles * (s / 2) >= kFullGrid) s /= 2;
+    return s;
+}
+// Blocks per thread of the block kernel: four (64-row tiles: half the staging
+// and parameter loads per pixel, about 7 % per row) unless the image's last tile
+// row would waste more than that or the launch would be small (512^2, 720
+// angles: 49 against 51.5 us; 700^2: 123 against 117; 361^2: 14.2 against 12.5).
+int blocks_for(int N, int split) {
+    const int rows4 = 64 * blk_tiles_y(N, 4), rows2 = 32 * blk_tiles_y(N, 2);
+    return 100 * rows2 >= 93 * rows4 && back_tiles_x(N) * blk_tiles_y(N, 4) * split >= kFullGrid ? 4 : 2;
 }
 }  // namespace
+
 bool ctg_back_blocks_ok(const BackAngle *host_tab, int n_angles) {
     for (int a = 0; a < n_angles; ++a)
         if (!(fabsf(host_tab[a].cf) <= 1.0f && fabsf(host_tab[a].sf) <= 1.0f)) return false;
@@ -587,59 +600,81 @@ bool ctg_back_blocks_ok(const BackAngle *host_tab, int n_angles) {
 
 namespace {
 
-template <typename T, int kChunk>
-void launch_back_tiled(const T *b, ColRef bc, int N, int n_angles, int n_det, const BackAngle *tab,
-                       int window, const float *add, float *x, cudaStream_t st) {
-    const size_t smem = back_smem(kChunk, window);
-    const dim3 grid(back_tiles_x(N), back_tiles_y(N), kPairSplit);
-    pixel_back_tiled_kernel<T, kChunk><<<grid, kPairThreads, smem, st>>>(b, bc, N, n_angles, n_det, tab, window, add,
-                                                                      x);
+// The arguments of one back projection.
+template <typename T> struct BackArgs {
+    const T *b;
+    ColRef bc;
+    int N, n_angles, n_det;
+    const BackAngle *tab;
+    int window;
+    const MatchedAngle *mt;
+    float thr;
+    const float *add;
+    float *x;
+    cudaStream_t st;
+};
+
+template <int kModel, int kChunk, int kRows, int kSplit, typename T>
+void launch_pair(const BackArgs<T> &a) {
+    const dim3 grid(back_tiles_x(a.N), back_tiles_y(a.N), kSplit);
+    pixel_pair_kernel<T, kModel, kChunk, kRows, kSplit>
+        <<<grid, pair_threads<kRows>(), pair_smem(kChunk, a.window), a.st>>>(
+            a.b, a.bc, a.N, a.n_angles, a.n_det, a.tab, a.window, a.mt, a.thr, a.add, a.x);
+}
+
+template <int kNB, int kSplit, typename T>
+void launch_blocks(const BackArgs<T> &a) {
+    const dim3 grid(back_tiles_x(a.N), blk_tiles_y(a.N, kNB), kSplit);
+    pixel_back_blocks_kernel<T, kNB, kSplit><<<grid, kBlkThreads, blk_smem(kNB), a.st>>>(
+        a.b, a.bc, a.N, a.n_angles, a.n_det, a.tab, a.add, a.x);
 }
 
 // blocks: the 2 x 2 block kernel (ctg_back_blocks_ok).  back_chunk: angles
-// staged per pass (16, 32 or 64) of the one-pixel tiled kernel.  Each pixel sums
-// its angles in the same order whatever the chunk, so the result does not
-// depend on it.
+// staged per pass of the one-pixel tiled kernel, 16 or (any other value, where
+// it fits) 32.  Each pixel sums its angles in the same order whatever the
+// chunk, so the result does not depend on it.
 template <typename T>
-cudaError_t launch_back_t(const T *b, ColRef bc, int N, int n_angles, int n_det, const BackAngle *tab,
-                          int window, bool blocks, const float *add, float *x, cudaStream_t st, int back_chunk) {
+cudaError_t launch_back_t(const BackArgs<T> &a, bool blocks, int back_chunk) {
     if (blocks) {
-        const int nb = blk_nb(N);
-        const dim3 grid(back_tiles_x(N), blk_tiles_y(N, nb), kPairSplit);
-        if (nb == 4)
-            pixel_back_blocks_kernel<T, 4><<<grid, kBlkThreads, blk_smem(4), st>>>(b, bc, N, n_angles, n_det, tab, add, x);
-        else
-            pixel_back_blocks_kernel<T, 2><<<grid, kBlkThreads, blk_smem(2), st>>>(b, bc, N, n_angles, n_det, tab, add, x);
-    } else if (window > 0 && window <= kBackWindowMaxTiled) {
-        const int chunk = back_chunk_for(back_chunk, window);
-        if (chunk == 64) launch_back_tiled<T, 64>(b, bc, N, n_angles, n_det, tab, window, add, x, st);
-        else if (chunk == 16) launch_back_tiled<T, 16>(b, bc, N, n_angles, n_det, tab, window, add, x, st);
-        else if (chunk == 8) launch_back_tiled<T, 8>(b, bc, N, n_angles, n_det, tab, window, add, x, st);
-        else launch_back_tiled<T, kPairChunk>(b, bc, N, n_angles, n_det, tab, window, add, x, st);
+        const int split = split_for(a.n_angles, back_tiles_x(a.N) * blk_tiles_y(a.N, 2));
+        const bool four = blocks_for(a.N, split) == 4;
+        if (split == 8) four ? launch_blocks<4, 8>(a) : launch_blocks<2, 8>(a);
+        else if (split == 4) four ? launch_blocks<4, 4>(a) : launch_blocks<2, 4>(a);
+        else four ? launch_blocks<4, 2>(a) : launch_blocks<2, 2>(a);
+    } else if (a.window > 0 && a.window <= kBackWindowMaxTiled) {
+        // four rows per thread (a finer pitch's windows leave room for few
+        // CTAs); two CTAs per cluster once that fills the device (pitch 0.75:
+        // 512^2, 1000 angles 138 us with 8, 1024^2 408 with 2 against 467 with 8)
+        const int chunk = back_chunk_for(back_chunk, a.window);
+        const bool two = back_tiles_x(a.N) * back_tiles_y(a.N) * 2 >= 2 * kFullGrid;
+        if (chunk == 8) two ? launch_pair<0, 8, 4, 2>(a) : launch_pair<0, 8, 4, 8>(a);
+        else if (chunk == 16) two ? launch_pair<0, 16, 4, 2>(a) : launch_pair<0, 16, 4, 8>(a);
+        else two ? launch_pair<0, kPairChunk, 4, 2>(a) : launch_pair<0, kPairChunk, 4, 8>(a);
     } else {
-        dim3 grid((N + kBX - 1) / kBX, (N + kBY - 1) / kBY);
-        pixel_back_kernel<T><<<grid, dim3(kBX, kBY), 0, st>>>(b, bc, N, n_angles, n_det, tab, add, x);
+        dim3 grid((a.N + kBX - 1) / kBX, (a.N + kBY - 1) / kBY);
+        pixel_back_kernel<T><<<grid, dim3(kBX, kBY), 0, a.st>>>(a.b, a.bc, a.N, a.n_angles, a.n_det, a.tab, a.add,
+                                                                a.x);
     }
     return cudaGetLastError();
 }
 
+// A^T or B_tau: four rows per thread (256 threads, more warps) for small
+// launches, eight (half the parameter loads and weights) from about six CTAs
+// per SM on (A^T, 200^2, 1000 angles: 35 against 41 us; 1001^2, 900 angles: 302
+// against 280); four CTAs per cluster for few angles.
+template <int kModel, int kChunk, typename T>
+void launch_matched(const BackArgs<T> &a) {
+    const int tiles = back_tiles_x(a.N) * back_tiles_y(a.N);
+    if (tiles * kMaxSplit < 2 * kFullGrid) launch_pair<kModel, kChunk, 4, 8>(a);
+    else if (split_for(a.n_angles, tiles) == kMaxSplit) launch_pair<kModel, kChunk, 8, 8>(a);
+    else launch_pair<kModel, kChunk, 8, 4>(a);
+}
+
 template <typename T>
-cudaError_t launch_matched_tiled_t(const T *b, ColRef bc, int N, int n_angles, int n_det,
-                                   const BackAngle *tab, int window, const MatchedAngle *mt, float thr,
-                                   const float *add, float *x, cudaStream_t st) {
-    const int chunk = std::min(kPairChunk, back_chunk_for(kPairChunk, window));
-    const size_t smem = back_smem(chunk, window);
-    const dim3 grid(back_tiles_x(N), back_tiles_y(N), kPairSplit);
-    auto run = [&](auto kernel) {
-        kernel<<<grid, kPairThreads, smem, st>>>(b, bc, N, n_angles, n_det, tab, window, mt, thr, add, x);
-    };
-    if (chunk == kPairChunk) {
-        if (thr > 0.0f) run(matched_back_tiled_kernel<T, 2, kPairChunk>);
-        else run(matched_back_tiled_kernel<T, 1, kPairChunk>);
-    } else {
-        if (thr > 0.0f) run(matched_back_tiled_kernel<T, 2, 16>);
-        else run(matched_back_tiled_kernel<T, 1, 16>);
-    }
+cudaError_t launch_matched_tiled_t(const BackArgs<T> &a) {
+    const bool full = back_chunk_for(kPairChunk, a.window) == kPairChunk;
+    if (a.thr > 0.0f) full ? launch_matched<2, kPairChunk>(a) : launch_matched<2, 16>(a);
+    else full ? launch_matched<1, kPairChunk>(a) : launch_matched<1, 16>(a);
     return cudaGetLastError();
 }
 
@@ -650,16 +685,14 @@ cudaError_t ctg_launch_back_matched_tiled(const void *b, int dtype, int N, int n
                                           float thr, const float *add, float *x, cudaStream_t st,
                                           ColRef bc) {
     if (window <= 0 || window > ctg_back_window_max()) return cudaErrorInvalidValue;
+    auto run = [&](auto *p) {
+        using T = typename std::remove_const<typename std::remove_pointer<decltype(p)>::type>::type;
+        return launch_matched_tiled_t(BackArgs<T>{p, bc, N, n_angles, n_det, tab, window, mt, thr, add, x, st});
+    };
     switch (dtype) {
-        case CTG_BASIS_FP32:
-            return launch_matched_tiled_t(static_cast<const float *>(b), bc, N, n_angles, n_det, tab, window,
-                                          mt, thr, add, x, st);
-        case CTG_BASIS_BF16:
-            return launch_matched_tiled_t(static_cast<const __nv_bfloat16 *>(b), bc, N, n_angles, n_det, tab,
-                                          window, mt, thr, add, x, st);
-        case CTG_BASIS_FP16:
-            return launch_matched_tiled_t(static_cast<const __half *>(b), bc, N, n_angles, n_det, tab, window,
-                                          mt, thr, add, x, st);
+        case CTG_BASIS_FP32: return run(static_cast<const float *>(b));
+        case CTG_BASIS_BF16: return run(static_cast<const __nv_bfloat16 *>(b));
+        case CTG_BASIS_FP16: return run(static_cast<const __half *>(b));
         default: return cudaErrorInvalidValue;
     }
 }
@@ -667,16 +700,15 @@ cudaError_t ctg_launch_back_matched_tiled(const void *b, int dtype, int N, int n
 cudaError_t ctg_launch_back(const void *b, int dtype, int N, int n_angles, int n_det,
                             const BackAngle *tab, int window, bool blocks, const float *add, float *x,
                             cudaStream_t st, int back_chunk, ColRef bc) {
+    auto run = [&](auto *p) {
+        using T = typename std::remove_const<typename std::remove_pointer<decltype(p)>::type>::type;
+        return launch_back_t(BackArgs<T>{p, bc, N, n_angles, n_det, tab, window, nullptr, 0.0f, add, x, st}, blocks,
+                             back_chunk);
+    };
     switch (dtype) {
-        case CTG_BASIS_FP32:
-            return launch_back_t(static_cast<const float *>(b), bc, N, n_angles, n_det, tab, window, blocks, add, x,
-                                 st, back_chunk);
-        case CTG_BASIS_BF16:
-            return launch_back_t(static_cast<const __nv_bfloat16 *>(b), bc, N, n_angles, n_det, tab, window,
-                                 blocks, add, x, st, back_chunk);
-        case CTG_BASIS_FP16:
-            return launch_back_t(static_cast<const __half *>(b), bc, N, n_angles, n_det, tab, window, blocks, add,
-                                 x, st, back_chunk);
+        case CTG_BASIS_FP32: return run(static_cast<const float *>(b));
+        case CTG_BASIS_BF16: return run(static_cast<const __nv_bfloat16 *>(b));
+        case CTG_BASIS_FP16: return run(static_cast<const __half *>(b));
         default: return cudaErrorInvalidValue;
     }
 }

@@ -104,3 +104,35 @@ def test_sixteen_bit_basis_column(P, oracle_mod):
         h = r.hessenberg(g, "ab", 1).cpu().numpy()[:, 0]
         q = oracle_mod.forward(og, oracle_mod.backproject(og, W[0]).reshape(50, 50))
         assert np.linalg.norm(q - W.T @ h) <= 2 * u * np.linalg.norm(q)
+
+
+@pytest.mark.parametrize("geom", [(47, 70, 100, 0, 180, 0.7), (1030, 40, 2100, 0, 180, 0.75)])
+def test_staged_chunk_does_not_change_the_result(P, oracle_mod, geom):
+    """Pitches below a pixel, 16 or 32 angles staged per pass, with eight and
+    with two CTAs per tile."""
+    import torch
+    g, og = P.Geometry(*geom), oracle_mod.Geometry(*geom)
+    b = np.random.default_rng(10).standard_normal(g.m).astype(np.float32)
+    bt = torch.tensor(b, device="cuda")
+    ctx = P.Context.get(bt.device)
+    try:
+        outs = []
+        for chunk in (16, 32, 64):
+            ctx.set_tiles(8, chunk)
+            outs.append(P.backproject(g, bt))
+    finally:
+        ctx.set_tiles(0, 0)
+    assert torch.equal(outs[0], outs[1]) and torch.equal(outs[1], outs[2])
+    ref = oracle_mod.backproject(og, b.astype(np.float64))
+    assert np.linalg.norm(outs[0].double().cpu().numpy() - ref) <= TOL * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("N,Na", [(1024, 60), (1024, 130), (700, 50), (512, 250)])
+def test_few_angles_take_smaller_clusters(P, oracle_mod, N, Na):
+    import torch
+    Nd = int(np.ceil(np.sqrt(2) * N))
+    g, og = P.Geometry(N, Na, Nd), oracle_mod.Geometry(N, Na, Nd)
+    b = np.random.default_rng(11).standard_normal(g.m).astype(np.float32)
+    got = P.backproject(g, torch.tensor(b, device="cuda")).double().cpu().numpy()
+    ref = oracle_mod.backproject(og, b.astype(np.float64))
+    assert np.linalg.norm(got - ref) <= TOL * np.linalg.norm(ref)
