@@ -94,8 +94,8 @@ void build_tables(const ctg_geom *g, std::vector<FwdAngle> &fw, std::vector<Back
         f.qf = (float)Q;
         f.df = (float)D;
         f.scale = (float)(1.0 / std::fabs(c));
-        f.row_driven = rd;
-        f.pad_ = 0;
+        f.row_group8 = rd ? 1u : 0u;
+        f.group4 = 0;
         BackAngle &b = bk[a];
         b.COS = to_fx(cs / ds);
         b.SIN = to_fx(sn / ds);
@@ -103,6 +103,7 @@ void build_tables(const ctg_geom *g, std::vector<FwdAngle> &fw, std::vector<Back
         b.cf = (float)(cs / ds);
         b.sf = (float)(sn / ds);
     }
+    ctg_forward_groups(fw);
 }
 
 // Per-angle weights of the matched back projector; *rm = the extra detector
@@ -155,8 +156,8 @@ struct GeomEntry {
     int rm = 0;
     float thr = 0.0f;           // B_tau threshold tau * max(A) (0: A^T)
     int *fwd_order = nullptr;   // forward dispatch orders of the shapes, one after another
-    size_t fwd_order_off[kFwdShapes] = {};
-    bool fwd_split_ok = false;  // shapes with several angles per warp are safe here
+    size_t fwd_order_off[kFwdShapes + 1] = {};
+    FwdGroups fwd_groups{};     // angle groups of the shapes, and where several angles per warp are safe
     int fwd_shape = 0;          // tile shapes in use (autotuned unless forced)
     int back_chunk = 32;
     bool tuned = false;
@@ -165,6 +166,10 @@ struct GeomEntry {
     unsigned long long last_use = 0;
     unsigned long long serial = 0;   // identifies the entry's device tables (graphs captured with them)
     const int *order_for(int shape) const { return fwd_order ? fwd_order + fwd_order_off[shape] : nullptr; }
+    int groups_for(int shape) const { return fwd_groups.count[fwd_split_index(kFwdShapeSplit[shape])]; }
+    bool split_ok(int split) const { return fwd_groups.safe[fwd_split_index(split)]; }
+    // the shape of two-image projections: eight angles per warp where safe
+    int two_shape() const { return split_ok(8) ? kFwdShapeTwo : fwd_shape; }
 };
 
 // x = B b (+ add) with the geometry's back projector; b of type `btype`
@@ -358,7 +363,7 @@ constexpr size_t kMaxCachedGeoms = 64;
 // one lane over its own chord in a fixed accumulator order; pixel-driven
 // back projection: angles staged per pass, each pixel's angles still in
 // order), so the choice changes the speed only.  Shapes with several angles
-// per warp are timed only where the geometry allows them (fwd_split_ok).  Each candidate is timed
+// per warp are timed only where the geometry allows them (split_ok).  Each candidate is timed
 // with CUDA events over 3 launches (after one untimed) on zero inputs of the
 // geometry's sizes on a private stream; the fastest is kept.
 int tune_geometry(GeomEntry *ge) {
@@ -390,11 +395,11 @@ int tune_geometry(GeomEntry *ge) {
     };
     for (int c = 0; c < kFwdShapes; ++c) {
         ge->fwd_us[c] = 0.0f;
-        if (kFwdShapeSplit[c] > 1 && !ge->fwd_split_ok) continue;
+        if (!ge->split_ok(kFwdShapeSplit[c])) continue;
         timed([&] {
             if (err == cudaSuccess)
                 err = ctg_launch_forward(pad, g->N, ge->pl, g->n_angles, g->n_det, ge->fwd, bv, st, c,
-                                         ge->order_for(c));
+                                         ge->groups_for(c), ge->order_for(c));
         }, &ge->fwd_us[c]);
     }
     const int back_cand[3] = {16, 32, 64};
@@ -444,7 +449,7 @@ int apply_tiles(ctg_ctx *ctx, GeomEntry *ge) {
         // a forced shape with several angles per warp falls back to one
         // angle per warp where the geometry does not allow it
         int split = ctx->force_fwd_angles ? ctx->force_fwd_split : 1;
-        if (split > 1 && !ge->fwd_split_ok) split = 1;
+        if (!ge->split_ok(split)) split = 1;
         int angles = ctx->force_fwd_angles ? ctx->force_fwd_angles : 8;
         if (split == 1) angles = std::min(angles, 8);
         ge->fwd_shape = 0;
@@ -486,6 +491,7 @@ int get_geom(ctg_ctx *ctx, const ctg_geom *g, GeomEntry **out) {
     std::vector<BackAngle> bk;
     build_tables(g, fw, bk);
     GeomEntry e;
+    e.fwd_groups = ctg_forward_groups(fw);
     e.g = *g;
     e.last_use = ++ctx->tick;
     e.serial = e.last_use;
@@ -499,12 +505,17 @@ int get_geom(ctg_ctx *ctx, const ctg_geom *g, GeomEntry **out) {
     if (err == cudaSuccess)
         err = cudaMemcpy(e.back, bk.data(), sizeof(BackAngle) * bk.size(), cudaMemcpyHostToDevice);
     if (err == cudaSuccess) {
-        e.fwd_split_ok = ctg_forward_split_safe(fw.data(), g->N, g->n_angles, g->n_det, e.pl, 4);
-        std::vector<int> all, o;
-        for (int c = 0; c < kFwdShapes; ++c) {
+        std::vector<int> orders[kFwdShapes + 1], all;
+        std::vector<int2> ranges;
+        ctg_forward_plan(fw.data(), g->N, g->n_angles, g->n_det, e.pl, 1, e.fwd_groups,
+                         {kFwdShapeWarps[0], kFwdShapeWarps[1]}, orders);
+        ctg_forward_plan(fw.data(), g->N, g->n_angles, g->n_det, e.pl, 4, e.fwd_groups,
+                         {kFwdShapeWarps[2], kFwdShapeWarps[3]}, orders + 2, &ranges);
+        ctg_forward_plan(fw.data(), g->N, g->n_angles, g->n_det, e.pl, 8, e.fwd_groups,
+                         {kFwdShapeWarps[kFwdShapeTwo]}, orders + kFwdShapeTwo, &ranges);
+        for (int c = 0; c <= kFwdShapes; ++c) {
             e.fwd_order_off[c] = all.size();
-            ctg_forward_order(fw.data(), g->N, g->n_angles, g->n_det, c, o);
-            all.insert(all.end(), o.begin(), o.end());
+            all.insert(all.end(), orders[c].begin(), orders[c].end());
         }
         err = cudaMalloc(&e.fwd_order, sizeof(int) * all.size());
         if (err == cudaSuccess)
@@ -670,7 +681,7 @@ struct SolveCtx {
         if (e != cudaSuccess) return e;
         return traced(ctx, 0, 1, st, [&] {
             return ctg_launch_forward(pad(), g->N, ge->pl, g->n_angles, g->n_det, ge->fwd, b, st,
-                                      ge->fwd_shape, ge->order_for(ge->fwd_shape));
+                                      ge->fwd_shape, ge->groups_for(ge->fwd_shape), ge->order_for(ge->fwd_shape));
         });
     }
     // b = A x and b2 = A x2 in one walk (x: column xc of the basis)
@@ -681,8 +692,9 @@ struct SolveCtx {
         });
         if (e != cudaSuccess) return e;
         return traced(ctx, 0, 1, st, [&] {
-            return ctg_launch_forward2(p4, g->N, ge->pl, g->n_angles, g->n_det, ge->fwd, b, b2, st,
-                                       ge->fwd_shape, ge->order_for(ge->fwd_shape));
+            const int c = ge->two_shape();
+            return ctg_launch_forward2(p4, g->N, ge->pl, g->n_angles, g->n_det, ge->fwd, b, b2, st, c,
+                                       ge->groups_for(c), ge->order_for(c));
         }, 2);
     }
     cudaError_t back(const void *b, const float *add, float *x, int btype = CTG_BASIS_FP32,
@@ -1401,7 +1413,7 @@ int ctg_project(ctg_ctx *ctx, const ctg_geom *g, const float *x_dev, float *b_de
     }));
     CTG_CK(traced(ctx, 0, 1, st, [&] {
         return ctg_launch_forward(ge->pad, g->N, ge->pl, g->n_angles, g->n_det, ge->fwd, b_dev, st,
-                                  ge->fwd_shape, ge->order_for(ge->fwd_shape));
+                                  ge->fwd_shape, ge->groups_for(ge->fwd_shape), ge->order_for(ge->fwd_shape));
     }));
     return CTG_OK;
 }

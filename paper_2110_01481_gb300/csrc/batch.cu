@@ -22,12 +22,12 @@ size_t al256(size_t v) { return (v + 255) & ~(size_t)255; }
 size_t rup(size_t v, size_t m) { return (v + m - 1) / m * m; }
 int padded4(int G) { return (G + 3) & ~3; }
 
-// Forward projector plan of a geometry: whether warps of several angles
-// are safe for it, and the dispatch orders (longest walk first) of its
-// blocks in the batched shapes 0 and kBatchFwdSplitShape.
+// Forward projector plan of a geometry: its angle groups and where warps of
+// several angles are safe, and the dispatch orders (longest walk first) of
+// blocks of kBatchFwdWarps warps with one, four and eight angles each.
 struct FwdPlan {
-    bool split_ok = false;
-    std::vector<int> order[2];
+    FwdGroups groups{};
+    std::vector<int> order[3];
 };
 
 struct InstPlan {
@@ -48,13 +48,26 @@ bool same_fwd_geom(const ctg_geom &a, const ctg_geom &b) {
 }
 
 // Forward projector plan of a geometry, from its host angle table.
-std::shared_ptr<const FwdPlan> plan_forward(const ctg_geom &g, const std::vector<FwdAngle> &fw) {
+std::shared_ptr<const FwdPlan> plan_forward(const ctg_geom &g, std::vector<FwdAngle> &fw) {
     auto f = std::make_shared<FwdPlan>();
     const PadLayout pl = ctg_pad_layout(g.N, g.det_spacing);
-    f->split_ok = ctg_forward_split_safe(fw.data(), g.N, g.n_angles, g.n_det, pl, 4);
-    ctg_forward_order(fw.data(), g.N, g.n_angles, g.n_det, 0, f->order[0]);
-    ctg_forward_order(fw.data(), g.N, g.n_angles, g.n_det, kBatchFwdSplitShape, f->order[1]);
+    f->groups = ctg_forward_groups(fw);
+    std::vector<int2> ranges;
+    for (const int split : {1, 4, 8})
+        ctg_forward_plan(fw.data(), g.N, g.n_angles, g.n_det, pl, split, f->groups, {kBatchFwdWarps},
+                         &f->order[fwd_split_index(split)], &ranges);
     return f;
+}
+
+// Angles per warp of an instance's forward projections in its rounds: eight for
+// two images and four for one, where safe (and `several` angles are allowed).
+void set_fwd_split(InstPlan &p, bool several) {
+    const FwdGroups &G = p.fwd->groups;
+    const bool two = p.variant == CTG_BA && p.o.noise_norm > 0.0;
+    int split = 1;
+    if (several && !p.d.pad_clamp) split = two && G.safe[2] ? 8 : (G.safe[1] ? 4 : 1);
+    p.d.fwd_split = split;
+    p.d.fwd_groups = G.count[fwd_split_index(split)];
 }
 
 int ck(cudaError_t e) {
@@ -151,6 +164,7 @@ int upload_tables(InstPlan &p, cudaStream_t st) {
     std::vector<BackAngle> bk;
     ctg_build_tables(&p.g, fw, bk);
     if (!p.fwd) p.fwd = plan_forward(p.g, fw);
+    set_fwd_split(p, true);
     BatchInst &d = p.d;
     d.back_window = ctg_back_window(bk.data(), p.g.n_angles);
     B_CK(cudaMemcpyAsync((void *)d.fwd, fw.data(), sizeof(FwdAngle) * fw.size(), cudaMemcpyHostToDevice, st));
@@ -179,6 +193,15 @@ cudaError_t back_inst(const InstPlan &p, const float *b, const float *add, float
     const BatchInst &d = p.d;
     return ctg_batch_back_one(b, d.back_model, p.g.N, p.g.n_angles, p.g.n_det, d.back, d.back_window, d.mt,
                               d.back_thr, add, x, st);
+}
+
+// b = A x of one solve on its own (its start and exit), from the staged image
+cudaError_t forward_inst(const InstPlan &p, float *b, cudaStream_t st) {
+    const BatchInst &d = p.d;
+    const FwdGroups &G = p.fwd->groups;
+    const int shape = G.safe[1] ? 2 : 1;
+    return ctg_launch_forward(d.pad, p.g.N, ctg_pad_layout(p.g.N, p.g.det_spacing), p.g.n_angles, p.g.n_det, d.fwd, b,
+                              st, shape, G.count[fwd_split_index(kFwdShapeSplit[shape])]);
 }
 
 RedScratch scratch_of(const BatchInst &d) {
@@ -252,7 +275,6 @@ struct RoundSpec {
     int off[MB_COUNT], len[MB_COUNT];
     int max_window, max_maxit;
     int *d_active;
-    int fwd_shape_ab, fwd_shape_ba;   // forward shapes of the two forward launches
     int back_chunk;                   // angles staged per pass by the back projections (0: 32)
     // the fused step: its largest k (0: the batch takes the separate
     // passes only), and in device memory the barrier counter, the timeout
@@ -264,11 +286,8 @@ struct RoundSpec {
 };
 
 // Build the block maps of instances `ids` (indices into the instance array).
-// split_ab / split_ba: the AB / BA forward launch may take the shape with
-// several angles per warp (it does when every one of its instances allows it).
 template <typename Plans>
-void build_maps(const Plans &plans, const std::vector<int> &ids, std::vector<int2> &maps, RoundSpec &rs,
-                bool split_ab = true, bool split_ba = true) {
+void build_maps(const Plans &plans, const std::vector<int> &ids, std::vector<int2> &maps, RoundSpec &rs) {
     maps.clear();
     auto add = [&](int which, auto count) {
         rs.off[which] = (int)maps.size();
@@ -290,31 +309,15 @@ void build_maps(const Plans &plans, const std::vector<int> &ids, std::vector<int
         return is_ab(p) && p.o.basis_dtype == CTG_BASIS_FP16 ? ctg_back_tiles(p.g.N) : 0;
     });
     add(MB_PAD_AB, [&](const InstPlan &p) { return is_ab(p) ? ctg_pad_tiles(p.g.N) : 0; });
-    // one forward shape per forward launch: several angles per warp when
-    // every instance of the launch allows it
-    auto shape_for = [&](bool ab) {
-        bool split = false, any = false;
-        for (int i : ids)
-            if (is_ab(plans[i]) == ab) {
-                split = (any ? split : true) && plans[i].fwd && plans[i].fwd->split_ok;
-                any = true;
-            }
-        return any && split && (ab ? split_ab : split_ba) ? kBatchFwdSplitShape : 0;
-    };
-    rs.fwd_shape_ab = shape_for(true);
-    rs.fwd_shape_ba = shape_for(false);
     auto add_fwd = [&](int which, bool ab) {
-        const int fs = ab ? rs.fwd_shape_ab : rs.fwd_shape_ba;
         add(which, [&](const InstPlan &p) {
-            return is_ab(p) == ab ? ctg_fwd_shape_blocks(fs, p.g.n_angles, p.g.n_det) : 0;
+            return is_ab(p) == ab ? ctg_fwd_blocks(kBatchFwdWarps, p.d.fwd_split, p.d.fwd_groups, p.g.n_det) : 0;
         });
         // each instance's forward blocks longest first (the result is the
         // same in any order; the launch's tail is shorter)
         for (int t = rs.off[which]; t < rs.off[which] + rs.len[which]; ++t) {
             const InstPlan &p = plans[maps[t].x];
-            if (!p.fwd) continue;
-            const std::vector<int> &o = p.fwd->order[fs == kBatchFwdSplitShape ? 1 : 0];
-            if ((int)o.size() == ctg_fwd_shape_blocks(fs, p.g.n_angles, p.g.n_det)) maps[t].y = o[maps[t].y];
+            maps[t].y = p.fwd->order[fwd_split_index(p.d.fwd_split)][maps[t].y];
         }
     };
     add_fwd(MB_FWD_AB, true);
@@ -360,7 +363,7 @@ int fused_kcap_of(const RoundSpec &rs, int max_maxit) {
 unsigned round_signature(const RoundSpec &r) {
     unsigned sig = 0;
     for (int i = 0; i < MB_COUNT; ++i) sig |= (r.len[i] > 0 ? 1u : 0u) << i;
-    return sig | (unsigned)r.fwd_shape_ab << 16 | (unsigned)r.fwd_shape_ba << 20;
+    return sig;
 }
 
 // Enqueue one round's launches on st (ending it with the stopping rules;
@@ -382,7 +385,7 @@ cudaError_t enqueue_round(const RoundSpec &r, cudaStream_t st, int *loop_ctl = n
         e = ctg_batch_back(r.insts, map(MB_H16), r.len[MB_H16], r.max_window, st, CTG_BASIS_FP16, r.back_chunk);
     if (e == cudaSuccess) e = ctg_batch_pad(r.insts, map(MB_PAD_AB), r.len[MB_PAD_AB], CTG_AB, st);
     if (e == cudaSuccess)
-        e = ctg_batch_forward(r.insts, map(MB_FWD_AB), r.len[MB_FWD_AB], CTG_AB, st, r.fwd_shape_ab);
+        e = ctg_batch_forward(r.insts, map(MB_FWD_AB), r.len[MB_FWD_AB], CTG_AB, st);
     if (fused) {
         const int which[3] = {MB_CGSF, MB_CGSF_B16, MB_CGSF_H16};
         const int types[3] = {CTG_BASIS_FP32, CTG_BASIS_BF16, CTG_BASIS_FP16};
@@ -400,7 +403,7 @@ cudaError_t enqueue_round(const RoundSpec &r, cudaStream_t st, int *loop_ctl = n
     if (e == cudaSuccess) e = ctg_batch_iterate(r.insts, map(MB_ITER), r.len[MB_ITER], r.max_maxit, st);
     if (e == cudaSuccess) e = ctg_batch_pad(r.insts, map(MB_PAD_BA), r.len[MB_PAD_BA], CTG_BA, st);
     if (e == cudaSuccess)
-        e = ctg_batch_forward(r.insts, map(MB_FWD_BA), r.len[MB_FWD_BA], CTG_BA, st, r.fwd_shape_ba);
+        e = ctg_batch_forward(r.insts, map(MB_FWD_BA), r.len[MB_FWD_BA], CTG_BA, st);
     if (e == cudaSuccess) e = ctg_batch_residual(r.insts, map(MB_RES), r.len[MB_RES], st);
     if (e == cudaSuccess) {
         if (loop_ctl)
@@ -502,23 +505,29 @@ int capture_loop(const RoundSpec &r, cudaStream_t st, cudaStream_t bs, int *loop
 int tune_batch(ctg_batch *b, const std::vector<int> &ids, bool tune_fwd, bool tune_back, bool *split_ab,
                bool *split_ba, int *chunk) {
     const int n = b->n;
-    std::vector<BatchInst> hi(n);
-    for (int i = 0; i < n; ++i) {
-        hi[i] = b->inst[i].d;
-        hi[i].active = 1;
-        hi[i].k = 1;
+    // maps and instances with several angles per warp, and with one
+    std::vector<BatchInst> hi[2] = {std::vector<BatchInst>(n), std::vector<BatchInst>(n)};
+    std::vector<int2> m[2];
+    RoundSpec r[2] = {};
+    for (int one = 0; one < 2; ++one) {
+        for (int i = 0; i < n; ++i) {
+            set_fwd_split(b->inst[i], !one);
+            hi[one][i] = b->inst[i].d;
+            hi[one][i].active = 1;
+            hi[one][i].k = 1;
+        }
+        build_maps(b->inst, ids, m[one], r[one]);
     }
-    B_CK(cudaMemcpy(b->d_insts, hi.data(), sizeof(BatchInst) * n, cudaMemcpyHostToDevice));
-    std::vector<int2> ms, mp;
-    RoundSpec rs{}, rp{};
-    build_maps(b->inst, ids, ms, rs, true, true);
-    build_maps(b->inst, ids, mp, rp, false, false);
+    const RoundSpec &rp = r[1];
     int2 *d = nullptr;
-    B_CK(cudaMalloc(&d, sizeof(int2) * (ms.size() + mp.size() + 1)));
-    int rc = ck(cudaMemcpy(d, ms.data(), sizeof(int2) * ms.size(), cudaMemcpyHostToDevice));
+    B_CK(cudaMalloc(&d, sizeof(int2) * (m[0].size() + m[1].size() + 1)));
+    int rc = ck(cudaMemcpy(d, m[0].data(), sizeof(int2) * m[0].size(), cudaMemcpyHostToDevice));
     if (rc == CTG_OK)
-        rc = ck(cudaMemcpy(d + ms.size(), mp.data(), sizeof(int2) * mp.size(), cudaMemcpyHostToDevice));
-    const int2 *ds = d, *dp = d + ms.size();
+        rc = ck(cudaMemcpy(d + m[0].size(), m[1].data(), sizeof(int2) * m[1].size(), cudaMemcpyHostToDevice));
+    const int2 *ds = d, *dp = d + m[0].size();
+    auto upload = [&](int one) {
+        if (rc == CTG_OK) rc = ck(cudaMemcpy(b->d_insts, hi[one].data(), sizeof(BatchInst) * n, cudaMemcpyHostToDevice));
+    };
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (rc == CTG_OK) rc = ck(cudaEventCreate(&e0));
     if (rc == CTG_OK) rc = ck(cudaEventCreate(&e1));
@@ -535,19 +544,20 @@ int tune_batch(ctg_batch *b, const std::vector<int> &ids, bool tune_fwd, bool tu
     };
     if (tune_fwd) {
         const int which[2] = {MB_FWD_AB, MB_FWD_BA}, variants[2] = {CTG_AB, CTG_BA};
-        const int shapes[2] = {rs.fwd_shape_ab, rs.fwd_shape_ba};
         bool *out[2] = {split_ab, split_ba};
-        for (int v = 0; v < 2; ++v) {
-            if (shapes[v] != kBatchFwdSplitShape || rs.len[which[v]] <= 0) continue;
-            const float t_split = timed([&] {
-                return ctg_batch_forward(b->d_insts, ds + rs.off[which[v]], rs.len[which[v]], variants[v], b->st,
-                                         kBatchFwdSplitShape);
-            });
-            const float t_one = timed([&] {
-                return ctg_batch_forward(b->d_insts, dp + rp.off[which[v]], rp.len[which[v]], variants[v], b->st, 0);
-            });
-            *out[v] = t_split <= t_one;
+        float t_us[2][2] = {};
+        for (int one = 0; one < 2; ++one) {
+            upload(one);
+            for (int v = 0; v < 2; ++v)
+                if (r[one].len[which[v]] > 0)
+                    t_us[v][one] = timed([&] {
+                        return ctg_batch_forward(b->d_insts, (one ? dp : ds) + r[one].off[which[v]],
+                                                 r[one].len[which[v]], variants[v], b->st);
+                    });
         }
+        for (int v = 0; v < 2; ++v) *out[v] = t_us[v][0] <= t_us[v][1];
+    } else {
+        upload(1);
     }
     if (tune_back && rp.len[MB_BACK] > 0) {
         float best = 0.0f;
@@ -566,6 +576,8 @@ int tune_batch(ctg_batch *b, const std::vector<int> &ids, bool tune_fwd, bool tu
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     cudaFree(d);
+    for (int i = 0; i < n; ++i)
+        set_fwd_split(b->inst[i], b->inst[i].variant == CTG_AB ? *split_ab : *split_ba);
     return rc;
 }
 
@@ -637,12 +649,14 @@ extern "C" int ctg_batch_create(ctg_ctx *ctx, int32_t n, const ctg_geom *geoms,
     ctg_ctx_forced_tiles(ctx, &f_split, &f_chunk);
     bool split_ab = f_split != 1, split_ba = f_split != 1;
     int chunk = f_chunk && ctg_batch_back_chunk_ok(f_chunk, b->max_window) ? f_chunk : 32;
+    if (rc == CTG_OK)
+        for (InstPlan &p : b->inst) set_fwd_split(p, p.variant == CTG_AB ? split_ab : split_ba);
     if (rc == CTG_OK && (!f_split || !f_chunk))
         rc = tune_batch(b, ids, !f_split, !f_chunk, &split_ab, &split_ba, &chunk);
     // block maps
     std::vector<int2> maps;
     RoundSpec spec{};
-    build_maps(b->inst, ids, maps, spec, split_ab, split_ba);
+    if (rc == CTG_OK) build_maps(b->inst, ids, maps, spec);
     spec.back_chunk = chunk;
     if (rc == CTG_OK) rc = ck(cudaMalloc(&b->d_maps, sizeof(int2) * (maps.empty() ? 1 : maps.size())));
     if (rc == CTG_OK && !maps.empty())
@@ -693,7 +707,7 @@ int enqueue_start(InstPlan &p, const float *b, const float *x0, double *stage, c
     if (d.pad2) B_CK(cudaMemsetAsync(d.pad2, 0, sizeof(float) * 2 * pl.floats, st));
     if (x0) {
         B_CK(ctg_launch_pad(x0, CTG_BASIS_FP32, d.pad, p.g.N, pl, st));
-        B_CK(ctg_launch_forward(d.pad, p.g.N, pl, p.g.n_angles, p.g.n_det, d.fwd, d.vm, st));
+        B_CK(forward_inst(p, d.vm, st));
     }
     if (p.variant == CTG_AB) {
         B_CK(ctg_sub_norm2(b, x0 ? d.vm : nullptr, d.vm, d.m, d.scal + 2, rs, st));
@@ -739,7 +753,7 @@ int activate(InstPlan &p, double *stage, ctg_info *info, cudaStream_t st, int *a
         // t_1 = A w_1, which the first round back-projects
         const PadLayout pl = ctg_pad_layout(p.g.N, p.g.det_spacing);
         B_CK(ctg_launch_pad(d.W, d.wtype, d.pad, p.g.N, pl, st));
-        B_CK(ctg_launch_forward(d.pad, p.g.N, pl, p.g.n_angles, p.g.n_det, d.fwd, d.vm, st));
+        B_CK(forward_inst(p, d.vm, st));
     }
     stage[6] = beta;
     B_CK(cudaMemcpyAsync(d.gg, &stage[6], sizeof(double), cudaMemcpyHostToDevice, st));
@@ -771,7 +785,7 @@ int enqueue_finish(const InstPlan &p, const BatchInst &d, const float *b, const 
         B_CK(ctg_gemv(d.W, d.wtype, d.ldw, d.n, k, d.y, x0, x, st));
     }
     B_CK(ctg_launch_pad(x, CTG_BASIS_FP32, d.pad, p.g.N, pl, st));
-    B_CK(ctg_launch_forward(d.pad, p.g.N, pl, p.g.n_angles, p.g.n_det, d.fwd, d.vm, st));
+    B_CK(forward_inst(p, d.vm, st));
     B_CK(ctg_sub_norm2(b, d.vm, nullptr, d.m, d.scal + 5, rs, st));
     B_CK(cudaMemcpyAsync(stage + 5, d.scal + 5, sizeof(double), cudaMemcpyDeviceToHost, st));
     if (info->history)

@@ -10,6 +10,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <initializer_list>
 #include <vector>
 
 #include "../../include/ctgmres.h"
@@ -23,13 +24,25 @@
 //   u(d, t) = Q + d * P + t * D,  P = ds / c,  Q = (h s - hd ds) / c + h,
 //   D = -s / c,  h = (N-1)/2,  hd = (n_det-1)/2,
 // and the ray sum is scaled by 1/|c|.  P, Q, D are 32.32 fixed point.
+//
+// A warp of the forward projector holds one, four or eight consecutive angles
+// that walk the same copy of the image.  The angles' groups for four and for
+// eight per warp are stored in the table itself: entry g's group word holds
+// group g's first angle and count (the groups are at most as many as the
+// angles).
 struct FwdAngle {
     long long P, Q, D;     // fixed point
     float pf, qf, df;      // the same in float, for the walk-range estimate
     float scale;           // 1 / |c|
-    int row_driven;        // 1: walk rows of x; 0: walk rows of x^T
-    int pad_;
+    unsigned row_group8;   // bit 0: row-driven (1: walk rows of x; 0: of x^T); bits 1-3: count - 1 of group g of
+                           // eight, bits 4-: its first angle
+    unsigned group4;       // bits 1-3, 4-: the same for groups of four
 };
+static inline unsigned fwd_group_word(int first, int count) { return (unsigned)first << 4 | (unsigned)(count - 1) << 1; }
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+static inline bool fwd_row_driven(const FwdAngle &t) { return t.row_group8 & 1u; }
 
 // Back-projection parameters of one angle: the detector position of pixel
 // (i, j) is u(i, j) = C + j * COS + i * SIN with COS = cos/ds, SIN = sin/ds,
@@ -106,41 +119,50 @@ cudaError_t ctg_launch_pad2(const void *x, int dtype, ColRef xc, const float *x2
 // per block x angles per warp (a warp holds 32 / angles-per-warp adjacent
 // rays of each of its angles).  Every shape gives the same result bit for
 // bit.  Shapes with several angles per warp are used only where
-// ctg_forward_split_safe holds for the geometry.
-constexpr int kFwdShapes = 4;
-constexpr int kFwdShapeAngles[kFwdShapes] = {8, 4, 8, 16};
-constexpr int kFwdShapeSplit[kFwdShapes] = {1, 1, 4, 4};
-// Forward shapes of batched launches: shape 0 (kBatchFwdAngles angles per
-// block, one per warp), or kBatchFwdSplitShape when every instance of the
-// round allows several angles per warp.
-constexpr int kBatchFwdAngles = 8;
-constexpr int kBatchFwdSplitShape = 3;
-// shape: an index into the tables above.  order: NULL, or the device copy
-// of ctg_forward_order's permutation for the same shape.
+// FwdGroups::safe holds for the geometry.  The last shape is not a candidate:
+// the projections of two images take it wherever eight angles per warp are
+// safe.
+constexpr int kFwdShapes = 4;                       // candidates
+constexpr int kFwdShapeTwo = 4;
+constexpr int kFwdShapeWarps[kFwdShapes + 1] = {8, 4, 2, 4, 1};
+constexpr int kFwdShapeSplit[kFwdShapes + 1] = {1, 1, 4, 4, 8};
+constexpr int kFwdShapeAngles[kFwdShapes + 1] = {8, 4, 8, 16, 8};
+// Blocks of batched forward launches have four warps, whatever an instance's
+// angles per warp (BatchInst::fwd_split): the shapes 1 and 3, or 32 angles.
+constexpr int kBatchFwdWarps = 4;
+// The groups of a geometry (index 0: one angle each, 1: four, 2: eight).
+struct FwdGroups {
+    int count[3];          // groups
+    bool safe[3];          // every lane of a warp stays inside the staged image's border
+};
+constexpr int fwd_split_index(int split) { return split == 8 ? 2 : (split == 4 ? 1 : 0); }
+// Writes the group words of the table (before it is used) and returns the
+// counts; `safe` is filled by ctg_forward_plan.
+FwdGroups ctg_forward_groups(std::vector<FwdAngle> &host_tab);
+// shape: an index into the tables above; ngroups: FwdGroups::count of its
+// angles per warp.  order: NULL, or the device copy of ctg_forward_plan's
+// permutation for the same shape.
 cudaError_t ctg_launch_forward(const float2 *pad, int N, const PadLayout &pl, int n_angles,
                                int n_det, const FwdAngle *tab, float *b, cudaStream_t st,
-                               int shape = 0, const int *order = nullptr);
+                               int shape, int ngroups, const int *order = nullptr);
 // b = A x and b2 = A x2 in one walk, from the interleaved staging of
 // ctg_launch_pad2; each ray's sums equal ctg_launch_forward's bit for bit.
 cudaError_t ctg_launch_forward2(const float4 *pad2, int N, const PadLayout &pl, int n_angles, int n_det,
-                                const FwdAngle *tab, float *b, float *b2, cudaStream_t st, int shape = 0,
+                                const FwdAngle *tab, float *b, float *b2, cudaStream_t st, int shape, int ngroups,
                                 const int *order = nullptr);
-// Blocks of one forward launch of `shape`.
-int ctg_fwd_shape_blocks(int shape, int n_angles, int n_det);
-// Dispatch order of the forward projector's blocks of `shape` (tile index
-// by * gx + bx, bx the ray group and by the angle group): longest estimated
-// walk first, which shortens the tail of the launch where the chord
-// lengths, and so the blocks' run times, differ.  From the host copy of the
-// angle table.
-void ctg_forward_order(const FwdAngle *host_tab, int N, int n_angles, int n_det, int shape,
-                       std::vector<int> &order);
-// Whether every lane of a warp holding `split` angles stays inside the
-// staged image's border over its warp's whole walk (checked at both ends of
-// a walk a few steps wider than the kernel's, in the kernel's fixed point).
-// Adjacent angles of a fine angular sampling pass; widely spaced ones, whose
-// chords differ, may not.
-bool ctg_forward_split_safe(const FwdAngle *host_tab, int N, int n_angles, int n_det,
-                            const PadLayout &pl, int split);
+// Blocks of one forward launch with `warps` warps of `split` angles per block.
+int ctg_fwd_blocks(int warps, int split, int ngroups, int n_det);
+// Fills G.safe[fwd_split_index(split)] (checked at both ends of a walk a few
+// steps wider than the kernel's, in the kernel's fixed point) and, for each
+// warps[i] (warps per block), the dispatch order of the forward projector's
+// blocks (tile index by * gx + bx, bx the ray group and by the block's place
+// among the angle groups): longest estimated walk first, which shortens the
+// tail of the launch where the chord lengths, and so the blocks' run times,
+// differ.  From the host copy of the angle table.  ranges: filled by split 4
+// (the walks' row ranges) and read by split 8, which comes after it.
+void ctg_forward_plan(const FwdAngle *host_tab, int N, int n_angles, int n_det, const PadLayout &pl, int split,
+                      FwdGroups &G, std::initializer_list<int> warps, std::vector<int> *orders,
+                      std::vector<int2> *ranges = nullptr);
 // Detector-window width (in bins) that the tiled back projector stages per
 // angle, from the host copy of the angle table.
 int ctg_back_window(const BackAngle *host_tab, int n_angles);
@@ -381,6 +403,8 @@ struct BatchInst {
     int N, n_angles, n_det, variant;      // variant: CTG_AB / CTG_BA
     const FwdAngle *fwd;
     const BackAngle *back;
+    int fwd_split;        // angles per warp of its forward projections (1, 4 or 8)
+    int fwd_groups;       // their groups (FwdGroups::count)
     int back_window;
     int pad_stride, pad_border, pad_clamp;
     long long n, m, L;
@@ -440,15 +464,12 @@ bool ctg_batch_back_chunk_ok(int chunk, int max_window);
 // (variant CTG_BA).
 cudaError_t ctg_batch_pad(BatchInst *insts, const int2 *map, int nblocks, int variant, cudaStream_t st);
 // The forward projection: AB q = A t; BA t_{k+1} = A w_{k+1} and, with the
-// DP stop, A x_k in the same walk.  shape: 0, or kBatchFwdSplitShape when
-// every instance of the launch allows it (ctg_forward_split_safe); the
-// map's local blocks are that shape's.
-cudaError_t ctg_batch_forward(BatchInst *insts, const int2 *map, int nblocks, int variant, cudaStream_t st,
-                              int shape = 0);
+// DP stop, A x_k in the same walk.  The map's local blocks are those of
+// ctg_fwd_blocks(kBatchFwdWarps, ...) for the instance's angles per warp.
+cudaError_t ctg_batch_forward(BatchInst *insts, const int2 *map, int nblocks, int variant, cudaStream_t st);
 // Local block counts of one instance for the maps above.
 int ctg_back_tiles(int N);
 int ctg_pad_tiles(int N);
-int ctg_fwd_blocks(int n_angles, int n_det);
 int ctg_back_window_max();
 // the three CGS2 passes and the scaling for the instances in `map`, whose
 // basis has element type wtype

@@ -126,50 +126,64 @@ __device__ __forceinline__ float one_plus_frac(unsigned lo) {
     return __uint_as_float(__funnelshift_r(lo, 0x7Fu, 9));
 }
 
-constexpr int kFwdAngles = kBatchFwdAngles;   // angles per batched block, one per warp
-constexpr int kFwdDepth = 12;   // image loads in flight per lane (a multiple of 4): with warps of
-                                // 4 angles, 12 measured 7% faster than 8 and 3% faster than 16 at
-                                // 512^2 (with one angle per warp, 8 was 10% faster than 4)
-constexpr int kBatchFwdDepth = 8;   // the batched kernel holds both clamp variants: 8 needs no spills
-constexpr int kFwdDepth2 = 8;       // two images: 8 interleaved loads (16 B each) in flight per lane
+// Image loads in flight per lane (multiples of 4).  The compiler, left alone,
+// holds these kernels to 32 registers for occupancy and serialises the loads
+// behind their uses; the launch bounds below leave it 64 (one image) and 80 (two),
+// enough for the loads: the walk is bound by load latency, and 32 warps per SM
+// with 16 loads each beat 64 with about 6.  512^2, 720 angles, 4 angles per warp:
+// 67.4 -> 63.6 us; 512^2, 180 angles, one angle per warp: 37 -> 25; two images with
+// 4 angles per warp: 153 -> 123.
+constexpr int kFwdDepth = 16;
+constexpr int kFwdDepth2 = 12;      // two images: 16-byte loads
+constexpr int fwd_min_blocks(int warps, int imgs) { return (imgs == 2 ? 24 : 32) / warps; }
 
 // b[a * n_det + d] = scale_a * sum_t lerp(img_a[t, .], u(d, t)).
-// A block holds kAngles consecutive angles; each warp holds kSplit of them
-// and 32 / kSplit adjacent rays of each, and walks the union of its rays'
+// A warp holds group `group` of kSplit consecutive angles (fewer where the
+// drive changes: all walk the same copy of the image) and 32 / kSplit adjacent
+// rays of each, ray group bx, and walks the union of its rays'
 // chords' row ranges in lockstep, so each load instruction reads one image
-// row per angle.  The walk position is 32.32 fixed point with the row stride
+// row per angle: the angles' taps in one row fall on nearly the same pairs, so
+// a warp load touches few sectors.  Two images interleaved (16-byte pairs) are
+// bound by the L1 data path, where eight angles per warp do best (512^2, 720
+// angles: 123 us with 4, 89 with 8; 1001^2, 900 angles: 534 and 394).
+// The walk position is 32.32 fixed point with the row stride
 // folded into the step, so its high word is the staged-pair index and its
 // low word the interpolation weight.  A lane outside its own chord reads
 // zero pairs in the border (or, with kClamp, a clamped index into the
 // 2-pair border).  The walk starts at a multiple of 4 and step s adds into
 // accumulator s % 4, so a ray's sum depends on its own chord only: every
 // block shape, warp layout and load depth gives the same result bit for
-// bit.  kSplit > 1 needs the host's check (ctg_forward_split_safe) that
+// bit.  kSplit > 1 needs the host's check (FwdGroups::safe) that
 // every lane stays inside the border.
 // kImgs = 2 projects two images staged interleaved (pad_pairs_block<2>) in
 // the same walk, b from the first and b2 from the second: each ray's two
 // sums are the ones the one-image kernel gives for each image alone.
-template <bool kClamp, int kAngles = kFwdAngles, int kSplit = 1, int kDepth = kFwdDepth, int kImgs = 1>
-__device__ __forceinline__ void joseph_forward_block(const void *__restrict__ pad_in, int N,
-                                                     int stride, int border, int n_angles,
-                                                     int n_det, const FwdAngle *__restrict__ tab,
-                                                     float *__restrict__ b, float *__restrict__ b2,
-                                                     int bx, int by) {
+template <bool kClamp, int kSplit, int kImgs>
+__device__ __forceinline__ void joseph_forward_warp(const void *__restrict__ pad_in, int N,
+                                                    int stride, int border, int n_det,
+                                                    const FwdAngle *__restrict__ tab,
+                                                    float *__restrict__ b, float *__restrict__ b2,
+                                                    int bx, int group) {
     using E = typename std::conditional<kImgs == 2, float4, float2>::type;
-    constexpr int kRays = 32 / kSplit;
-    const int lane = threadIdx.x & 31;
-    const int a = by * kAngles + (threadIdx.x >> 5) * kSplit + lane / kRays;
-    const bool live = a < n_angles;
-    if (!__any_sync(0xffffffffu, live)) return;      // whole warp past the last angle
+    constexpr int kRays = 32 / kSplit, kDepth = kImgs == 2 ? kFwdDepth2 : kFwdDepth;
+    const int lane = threadIdx.x & 31, ai = lane / kRays;
+    int a = group, na = 1;
+    if constexpr (kSplit > 1) {
+        const unsigned g = kSplit == 8 ? tab[group].row_group8 : tab[group].group4;
+        a = (int)(g >> 4);
+        na = (int)((g >> 1) & 7u) + 1;
+        a += min(ai, na - 1);             // lanes past the group's last angle walk with it
+    }
     const int d = bx * kRays + lane % kRays;
-    const FwdAngle t = tab[live ? a : n_angles - 1];
-    const E *img = static_cast<const E *>(pad_in) + (t.row_driven ? 0 : (size_t)N * stride) + border;
+    const bool live = ai < na && d < n_det;
+    const FwdAngle t = tab[a];
+    const E *img = static_cast<const E *>(pad_in) + (fwd_row_driven(t) ? 0 : (size_t)N * stride) + border;
 
     // this ray's steps whose taps can touch the image (-1 < u < N), with a
     // one-step margin; rays past the last detector or angle take an empty
     // range
     int lo = N, hi = -1;
-    if (live && d < n_det) {
+    if (live) {
         const float u0 = fmaf((float)d, t.pf, t.qf);
         if (fabsf(t.df) > 1e-20f) {
             const float r1 = (-1.0f - u0) / t.df, r2 = ((float)N - u0) / t.df;
@@ -244,24 +258,25 @@ __device__ __forceinline__ void joseph_forward_block(const void *__restrict__ pa
             U += t.D;
         }
     }
-    if (live && d < n_det) {
+    if (live) {
         b[(size_t)a * n_det + d] = ((acc[0] + acc[2]) + (acc[1] + acc[3])) * t.scale;
         if constexpr (kImgs == 2) b2[(size_t)a * n_det + d] = ((acc[4] + acc[6]) + (acc[5] + acc[7])) * t.scale;
     }
 }
 
-// One block per (ray group bx, angle group by), on a 1-D grid of gx * gy
-// blocks; block i takes tile order[i] = by * gx + bx (order NULL: tile i),
+// One block per (ray group bx, kWarps angle groups by), on a 1-D grid of gx *
+// gy blocks; block i takes tile order[i] = by * gx + bx (order NULL: tile i),
 // so that the dispatch order can put the longest walks first.
-template <bool kClamp, int kAngles, int kSplit, int kImgs>
-__global__ void __launch_bounds__(32 * kAngles / kSplit)
-joseph_forward_kernel(const void *__restrict__ pad, int N, int stride, int border,
-                      int n_angles, int n_det, const FwdAngle *__restrict__ tab,
+template <bool kClamp, int kWarps, int kSplit, int kImgs>
+__global__ void __launch_bounds__(32 * kWarps, fwd_min_blocks(kWarps, kImgs))
+joseph_forward_kernel(const void *__restrict__ pad, int N, int stride, int border, int ngroups,
+                      int n_det, const FwdAngle *__restrict__ tab,
                       float *__restrict__ b, float *__restrict__ b2, const int *__restrict__ order,
                       int gx) {
     const int tile = order ? order[blockIdx.x] : (int)blockIdx.x;
-    joseph_forward_block<kClamp, kAngles, kSplit, kImgs == 2 ? kFwdDepth2 : kFwdDepth, kImgs>(
-        pad, N, stride, border, n_angles, n_det, tab, b, b2, tile % gx, tile / gx);
+    const int group = tile / gx * kWarps + (threadIdx.x >> 5);
+    if (group >= ngroups) return;                     // whole warp past the last group
+    joseph_forward_warp<kClamp, kSplit, kImgs>(pad, N, stride, border, n_det, tab, b, b2, tile % gx, group);
 }
 
 // ---------------------------------------------------------------------------
@@ -488,34 +503,32 @@ __global__ void batch_pad_kernel(const BatchInst *__restrict__ insts, const int2
     else stage(static_cast<const float *>(I.W));
 }
 
-// kAngles, kSplit: the forward shape of the launch (one for all instances).
 // AB: q = A t (into vm); BA: t_{k+1} = A w_{k+1} (into vm) and, with the DP
-// stop, A x_k (into vr) from the two-image staging.
-template <int kVariant, int kAngles, int kSplit>
-__global__ void __launch_bounds__(32 * kAngles / kSplit)
+// stop, A x_k (into vr) from the two-image staging.  Each instance has its own
+// angles per warp.
+template <int kImgs>
+__device__ __forceinline__ void batch_forward(const BatchInst &I, const void *pad, float *b2, int tile) {
+    const int rays = 32 / I.fwd_split, bxn = (I.n_det + rays - 1) / rays;
+    const int bx = tile % bxn, group = tile / bxn * kBatchFwdWarps + (threadIdx.x >> 5);
+    if (group >= I.fwd_groups) return;
+    if (I.pad_clamp)
+        joseph_forward_warp<true, 1, kImgs>(pad, I.N, I.pad_stride, I.pad_border, I.n_det, I.fwd, I.vm, b2, bx, group);
+    else if (kImgs == 2 && I.fwd_split == 8)
+        joseph_forward_warp<false, 8, kImgs>(pad, I.N, I.pad_stride, I.pad_border, I.n_det, I.fwd, I.vm, b2, bx, group);
+    else if (I.fwd_split == 4)
+        joseph_forward_warp<false, 4, kImgs>(pad, I.N, I.pad_stride, I.pad_border, I.n_det, I.fwd, I.vm, b2, bx, group);
+    else
+        joseph_forward_warp<false, 1, kImgs>(pad, I.N, I.pad_stride, I.pad_border, I.n_det, I.fwd, I.vm, b2, bx, group);
+}
+
+template <int kVariant>
+__global__ void __launch_bounds__(32 * kBatchFwdWarps, fwd_min_blocks(kBatchFwdWarps, kVariant == CTG_BA ? 2 : 1))
 batch_forward_kernel(const BatchInst *__restrict__ insts, const int2 *__restrict__ map) {
     const int2 mp = map[blockIdx.x];
     const BatchInst &I = insts[mp.x];
     if (!I.active) return;
-    const int bxn = (I.n_det + 32 / kSplit - 1) / (32 / kSplit);
-    const int bx = mp.y % bxn, by = mp.y / bxn;
-    if (kVariant == CTG_BA && I.target > 0.0) {
-        if (I.pad_clamp)
-            joseph_forward_block<true, kAngles, kSplit, kBatchFwdDepth, 2>(
-                I.pad2, I.N, I.pad_stride, I.pad_border, I.n_angles, I.n_det, I.fwd, I.vm, I.vr, bx, by);
-        else
-            joseph_forward_block<false, kAngles, kSplit, kBatchFwdDepth, 2>(
-                I.pad2, I.N, I.pad_stride, I.pad_border, I.n_angles, I.n_det, I.fwd, I.vm, I.vr, bx, by);
-        return;
-    }
-    if (I.pad_clamp)
-        joseph_forward_block<true, kAngles, kSplit, kBatchFwdDepth>(I.pad, I.N, I.pad_stride, I.pad_border,
-                                                                    I.n_angles, I.n_det, I.fwd, I.vm, nullptr,
-                                                                    bx, by);
-    else
-        joseph_forward_block<false, kAngles, kSplit, kBatchFwdDepth>(I.pad, I.N, I.pad_stride, I.pad_border,
-                                                                     I.n_angles, I.n_det, I.fwd, I.vm, nullptr,
-                                                                     bx, by);
+    if (kVariant == CTG_BA && I.target > 0.0) batch_forward<2>(I, I.pad2, I.vr, mp.y);
+    else batch_forward<1>(I, I.pad, nullptr, mp.y);
 }
 
 }  // namespace
@@ -528,10 +541,9 @@ int ctg_pad_tiles(int N) {
     const int t = (N + kPadTile - 1) / kPadTile;
     return t * t;
 }
-int ctg_fwd_blocks(int n_angles, int n_det) {
-    static_assert(kFwdShapeAngles[0] == kFwdAngles && kFwdShapeSplit[0] == 1, "batched forward shape");
-    static_assert(kFwdShapeSplit[kBatchFwdSplitShape] > 1, "batched split shape");
-    return ctg_fwd_shape_blocks(0, n_angles, n_det);
+int ctg_fwd_blocks(int warps, int split, int ngroups, int n_det) {
+    const int rays = 32 / split;
+    return ((n_det + rays - 1) / rays) * ((ngroups + warps - 1) / warps);
 }
 // largest window the tiled back projector can stage in shared memory
 int ctg_back_window_max() { return (40 * 1024) / (int)(sizeof(float2) * kBChunk); }
@@ -586,22 +598,10 @@ cudaError_t ctg_batch_pad(BatchInst *insts, const int2 *map, int nblocks, int va
     return cudaGetLastError();
 }
 
-namespace {
-template <int kVariant>
-void batch_forward_t(BatchInst *insts, const int2 *map, int nblocks, cudaStream_t st, int shape) {
-    constexpr int SA = kFwdShapeAngles[kBatchFwdSplitShape], SS = kFwdShapeSplit[kBatchFwdSplitShape];
-    if (shape == kBatchFwdSplitShape)
-        batch_forward_kernel<kVariant, SA, SS><<<nblocks, 32 * SA / SS, 0, st>>>(insts, map);
-    else
-        batch_forward_kernel<kVariant, kFwdAngles, 1><<<nblocks, 32 * kFwdAngles, 0, st>>>(insts, map);
-}
-}  // namespace
-
-cudaError_t ctg_batch_forward(BatchInst *insts, const int2 *map, int nblocks, int variant, cudaStream_t st,
-                              int shape) {
+cudaError_t ctg_batch_forward(BatchInst *insts, const int2 *map, int nblocks, int variant, cudaStream_t st) {
     if (nblocks <= 0) return cudaSuccess;
-    if (variant == CTG_AB) batch_forward_t<CTG_AB>(insts, map, nblocks, st, shape);
-    else batch_forward_t<CTG_BA>(insts, map, nblocks, st, shape);
+    if (variant == CTG_AB) batch_forward_kernel<CTG_AB><<<nblocks, 32 * kBatchFwdWarps, 0, st>>>(insts, map);
+    else batch_forward_kernel<CTG_BA><<<nblocks, 32 * kBatchFwdWarps, 0, st>>>(insts, map);
     return cudaGetLastError();
 }
 
@@ -660,32 +660,36 @@ cudaError_t ctg_launch_pad2(const void *x, int dtype, ColRef xc, const float *x2
 
 namespace {
 
-template <int kAngles, int kSplit, int kImgs>
-void launch_forward_t(const void *pad, int N, const PadLayout &pl, int n_angles, int n_det,
-                      const FwdAngle *tab, float *b, float *b2, cudaStream_t st, const int *order) {
-    constexpr int kRays = 32 / kSplit;
-    const int gx = (n_det + kRays - 1) / kRays, gy = (n_angles + kAngles - 1) / kAngles;
-    const unsigned grid = (unsigned)gx * (unsigned)gy;
+template <int kShape, int kImgs>
+void launch_forward_t(const void *pad, int N, const PadLayout &pl, int n_det, const FwdAngle *tab, float *b,
+                      float *b2, cudaStream_t st, int ngroups, const int *order) {
+    constexpr int kWarps = kFwdShapeWarps[kShape], kSplit = kFwdShapeSplit[kShape], kRays = 32 / kSplit;
+    const int gx = (n_det + kRays - 1) / kRays;
+    const unsigned grid = (unsigned)ctg_fwd_blocks(kWarps, kSplit, ngroups, n_det);
     if (pl.clamp)
-        joseph_forward_kernel<true, kAngles, kSplit, kImgs><<<grid, 32 * kAngles / kSplit, 0, st>>>(
-            pad, N, pl.stride, pl.border, n_angles, n_det, tab, b, b2, order, gx);
+        joseph_forward_kernel<true, kWarps, kSplit, kImgs><<<grid, 32 * kWarps, 0, st>>>(
+            pad, N, pl.stride, pl.border, ngroups, n_det, tab, b, b2, order, gx);
     else
-        joseph_forward_kernel<false, kAngles, kSplit, kImgs><<<grid, 32 * kAngles / kSplit, 0, st>>>(
-            pad, N, pl.stride, pl.border, n_angles, n_det, tab, b, b2, order, gx);
+        joseph_forward_kernel<false, kWarps, kSplit, kImgs><<<grid, 32 * kWarps, 0, st>>>(
+            pad, N, pl.stride, pl.border, ngroups, n_det, tab, b, b2, order, gx);
 }
 
 template <int kImgs>
-void launch_forward_shape(int shape, const void *pad, int N, const PadLayout &pl, int n_angles, int n_det,
-                          const FwdAngle *tab, float *b, float *b2, cudaStream_t st, const int *order) {
+void launch_forward_shape(int shape, const void *pad, int N, const PadLayout &pl, int n_det, const FwdAngle *tab,
+                          float *b, float *b2, cudaStream_t st, int ngroups, const int *order) {
     switch (shape) {
-        case 1: launch_forward_t<4, 1, kImgs>(pad, N, pl, n_angles, n_det, tab, b, b2, st, order); break;
-        case 2: launch_forward_t<8, 4, kImgs>(pad, N, pl, n_angles, n_det, tab, b, b2, st, order); break;
-        case 3: launch_forward_t<16, 4, kImgs>(pad, N, pl, n_angles, n_det, tab, b, b2, st, order); break;
-        default: launch_forward_t<8, 1, kImgs>(pad, N, pl, n_angles, n_det, tab, b, b2, st, order); break;
+        case 1: launch_forward_t<1, kImgs>(pad, N, pl, n_det, tab, b, b2, st, ngroups, order); break;
+        case 2: launch_forward_t<2, kImgs>(pad, N, pl, n_det, tab, b, b2, st, ngroups, order); break;
+        case 3: launch_forward_t<3, kImgs>(pad, N, pl, n_det, tab, b, b2, st, ngroups, order); break;
+        case kFwdShapeTwo:
+            if constexpr (kImgs == 2)
+                launch_forward_t<kFwdShapeTwo, 2>(pad, N, pl, n_det, tab, b, b2, st, ngroups, order);
+            break;
+        default: launch_forward_t<0, kImgs>(pad, N, pl, n_det, tab, b, b2, st, ngroups, order); break;
     }
 }
 
-// walk range [lo, hi] of ray d of angle t, as joseph_forward_block
+// walk range [lo, hi] of ray d of angle t, as joseph_forward_warp
 // estimates it (host arithmetic; may differ from the device's by a step).
 // Returns 0 for a ray that meets the image; for one that misses it (lo = N, hi
 // = -1), -1 or 1 as its crossing lies before the first or past the last row.
@@ -736,76 +740,109 @@ void group_range(const FwdAngle &t, int N, int d0, int d1, int &wlo, int &whi) {
 
 cudaError_t ctg_launch_forward(const float2 *pad, int N, const PadLayout &pl, int n_angles,
                                int n_det, const FwdAngle *tab, float *b, cudaStream_t st,
-                               int shape, const int *order) {
+                               int shape, int ngroups, const int *order) {
     // every ray's sum depends on its own chord only, so the result depends
     // on neither the shape nor the dispatch order
-    launch_forward_shape<1>(shape, pad, N, pl, n_angles, n_det, tab, b, nullptr, st, order);
+    (void)n_angles;
+    launch_forward_shape<1>(shape, pad, N, pl, n_det, tab, b, nullptr, st, ngroups, order);
     return cudaGetLastError();
 }
 
 cudaError_t ctg_launch_forward2(const float4 *pad2, int N, const PadLayout &pl, int n_angles, int n_det,
-                                const FwdAngle *tab, float *b, float *b2, cudaStream_t st, int shape,
+                                const FwdAngle *tab, float *b, float *b2, cudaStream_t st, int shape, int ngroups,
                                 const int *order) {
-    launch_forward_shape<2>(shape, pad2, N, pl, n_angles, n_det, tab, b, b2, st, order);
+    (void)n_angles;
+    launch_forward_shape<2>(shape, pad2, N, pl, n_det, tab, b, b2, st, ngroups, order);
     return cudaGetLastError();
 }
 
-int ctg_fwd_shape_blocks(int shape, int n_angles, int n_det) {
-    const int rays = 32 / kFwdShapeSplit[shape], angles = kFwdShapeAngles[shape];
-    return ((n_det + rays - 1) / rays) * ((n_angles + angles - 1) / angles);
-}
-
-void ctg_forward_order(const FwdAngle *tab, int N, int n_angles, int n_det, int shape,
-                       std::vector<int> &order) {
-    const int A = kFwdShapeAngles[shape], S = kFwdShapeSplit[shape], R = 32 / S;
-    const int gx = (n_det + R - 1) / R, gy = (n_angles + A - 1) / A;
-    // work of a tile: the steps of its warps' lockstep walks plus a fixed
-    // cost per warp
-    std::vector<long long> cost((size_t)gx * gy, 0);
-    for (int a0 = 0; a0 < n_angles; a0 += S)
-        for (int bx = 0; bx < gx; ++bx) {
-            int wlo = N, whi = -1;
-            for (int a = a0; a < std::min(n_angles, a0 + S); ++a) {
-                int lo, hi;
-                group_range(tab[a], N, bx * R, std::min(n_det, bx * R + R), lo, hi);
-                wlo = std::min(wlo, lo);
-                whi = std::max(whi, hi);
-            }
-            cost[(size_t)(a0 / A) * gx + bx] += (whi >= wlo ? whi - (wlo & ~3) + 1 : 0) + 16;
+FwdGroups ctg_forward_groups(std::vector<FwdAngle> &tab) {
+    FwdGroups G{};
+    const int n = (int)tab.size();
+    G.count[0] = n;
+    G.safe[0] = true;
+    for (int a = 0; a < n; ++a) {
+        tab[a].row_group8 &= 1u;
+        tab[a].group4 = 0;
+    }
+    for (const int split : {4, 8}) {
+        int &g = G.count[fwd_split_index(split)];
+        for (int a = 0, c; a < n; a += c, ++g) {
+            for (c = 1; c < split && a + c < n && fwd_row_driven(tab[a + c]) == fwd_row_driven(tab[a]);) ++c;
+            (split == 8 ? tab[g].row_group8 : tab[g].group4) |= fwd_group_word(a, c);
         }
-    order.resize(cost.size());
-    for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
-    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return cost[x] > cost[y]; });
+    }
+    return G;
 }
 
-bool ctg_forward_split_safe(const FwdAngle *tab, int N, int n_angles, int n_det, const PadLayout &pl,
-                            int split) {
-    if (pl.clamp) return true;                      // indices are clamped
-    const int R = 32 / split;
-    for (int a0 = 0; a0 < n_angles; a0 += split)
-        for (int d0 = 0; d0 < n_det; d0 += R) {
+namespace {
+// Block order, longest first (stable): a counting sort of the blocks' steps.
+void longest_first(const std::vector<int> &cost, int ng, int gx, int W, std::vector<int> &order) {
+    const int gy = (ng + W - 1) / W;
+    std::vector<int> sum((size_t)gx * gy, 0), at;
+    for (int g = 0; g < ng; ++g)
+        for (int bx = 0; bx < gx; ++bx) sum[(size_t)(g / W) * gx + bx] += cost[(size_t)g * gx + bx];
+    const int top = sum.empty() ? 0 : *std::max_element(sum.begin(), sum.end());
+    at.assign((size_t)top + 2, 0);
+    for (const int c : sum) ++at[top - c + 1];
+    for (int c = 0; c <= top; ++c) at[c + 1] += at[c];
+    order.resize(sum.size());
+    for (size_t i = 0; i < sum.size(); ++i) order[at[top - sum[i]]++] = (int)i;
+}
+}  // namespace
+
+void ctg_forward_plan(const FwdAngle *tab, int N, int n_angles, int n_det, const PadLayout &pl, int split,
+                      FwdGroups &G, std::initializer_list<int> warps, std::vector<int> *orders,
+                      std::vector<int2> *ranges) {
+    const int R = 32 / split, gx = (n_det + R - 1) / R, ng = G.count[fwd_split_index(split)];
+    // groups cut short by changes of drive leave lanes idle: not worth it when
+    // more than a fifth are (widely spaced angles)
+    bool safe = split == 1 || (long long)ng * split * 4 <= 5LL * n_angles + 12 * split;
+    // eight angles and four rays: from the ranges of the two groups of four
+    // (each group of eight is one or two of them) and their eight rays
+    const int gx4 = (n_det + 7) / 8;
+    if (split == 4) ranges->resize((size_t)ng * gx);
+    // steps of each warp's lockstep walk plus a fixed cost
+    std::vector<int> cost((size_t)ng * gx);
+    for (int g = 0, g4 = 0; g < ng; ++g) {
+        const unsigned w = split == 8 ? tab[g].row_group8 : tab[g].group4;
+        const int a0 = split == 1 ? g : (int)(w >> 4), na = split == 1 ? 1 : (int)((w >> 1) & 7u) + 1;
+        for (int bx = 0; bx < gx; ++bx) {
+            const int d0 = bx * R, d1 = std::min(n_det, d0 + R);
             int wlo = N, whi = -1;
-            for (int a = a0; a < std::min(n_angles, a0 + split); ++a) {
-                int lo, hi;
-                group_range(tab[a], N, d0, std::min(n_det, d0 + R), lo, hi);
-                wlo = std::min(wlo, lo);
-                whi = std::max(whi, hi);
+            if (split == 8) {
+                for (int h = 0; h < (na > 4 ? 2 : 1); ++h) {
+                    const int2 r = (*ranges)[(size_t)(g4 + h) * gx4 + bx / 2];
+                    wlo = std::min(wlo, r.x);
+                    whi = std::max(whi, r.y);
+                }
+            } else {
+                for (int a = a0; a < a0 + na; ++a) {
+                    int lo, hi;
+                    group_range(tab[a], N, d0, d1, lo, hi);
+                    wlo = std::min(wlo, lo);
+                    whi = std::max(whi, hi);
+                }
+                if (split == 4) (*ranges)[(size_t)g * gx + bx] = make_int2(wlo, whi);
             }
-            if (whi < wlo) continue;
+            cost[(size_t)g * gx + bx] = (whi >= wlo ? whi - (wlo & ~3) + 1 : 0) + 16;
+            if (!safe || split == 1 || pl.clamp || whi < wlo) continue;     // clamped indices are safe
             // the device's range may differ from this estimate by a step:
             // check a wider one
             const int s_lo = std::max(0, (wlo & ~3) - 4), s_hi = std::min(N - 1, whi + 4);
             // a lane's column is affine in its ray d, so the warp's first and
-            // last ray of each angle are its extremes (lanes past the last
-            // angle walk with the last angle's table)
-            for (int a = a0; a < a0 + split; ++a) {
-                const FwdAngle &t = tab[std::min(n_angles - 1, a)];
-                for (const long long d : {(long long)d0, (long long)(d0 + R - 1)})
-                    for (const long long s : {(long long)s_lo, (long long)s_hi}) {
-                        const long long j = (t.Q + d * t.P + s * t.D) >> CTG_FXF_BITS;
-                        if (j < -pl.border || j > N - 1 + pl.border) return false;
-                    }
+            // last ray of each angle are its extremes
+            long long least = 0, most = 0;
+            for (int a = a0; a < a0 + na; ++a) {
+                const long long u = tab[a].Q + d0 * tab[a].P + s_lo * tab[a].D;
+                const long long dd = (R - 1) * tab[a].P, ds = (s_hi - s_lo) * tab[a].D;
+                least = std::min(least, u + std::min(0LL, dd) + std::min(0LL, ds));
+                most = std::max(most, u + std::max(0LL, dd) + std::max(0LL, ds));
             }
+            if ((least >> CTG_FXF_BITS) < -pl.border || (most >> CTG_FXF_BITS) > N - 1 + pl.border) safe = false;
         }
-    return true;
+        g4 += na > 4 ? 2 : 1;
+    }
+    G.safe[fwd_split_index(split)] = safe;
+    for (const int W : warps) longest_first(cost, ng, gx, W, *orders++);
 }
