@@ -217,7 +217,9 @@ int ctg_workspace_layout(const ctg_geom *g, int variant, const ctg_opts *o,
 /* AB-GMRES (Sec. 2, left column): x = x0 + B W_k y_k.
  * b: m floats; x0: n floats or NULL (x0 = 0); x: n floats (output).
  * workspace: device memory of >= workspace_bytes bytes, 256-byte aligned, or
- * NULL, in which case the library allocates and frees it per call.  The
+ * NULL, in which case the library takes it from a memory pool of the
+ * context per call, in stream order (the pool keeps up to 512 MiB between
+ * calls, until ctg_destroy).  The
  * caller owns b, x0, x and the workspace; none may alias another.  Runs on
  * `stream`, synchronises it before returning and fills *info (info may not
  * be NULL).  A breakdown (h_{k+1,k} <= 1e-6 ||A B w_k||) is reported in
@@ -226,8 +228,8 @@ int ctg_workspace_layout(const ctg_geom *g, int variant, const ctg_opts *o,
  * Hessenberg least-squares problem, y_k and the stopping rule are device
  * kernels, and the whole solve is one CUDA graph (the start, while-loop
  * nodes over the steps, the exit) that the context captures on first use
- * and replays for later calls with the same pointers and options; the host
- * waits once, at the end.  With phase tracing on (ctg_set_timing) the same
+ * and replays for later calls with the same geometry, options and workspace,
+ * whatever b, x0, x, tau and noise_norm are; the host waits once, at the end.  With phase tracing on (ctg_set_timing) the same
  * kernels are enqueued step by step instead.  Returns CTG_ERR_TIMEOUT if a
  * bounded device-side wait gave up (ctg_set_wait_limit). */
 int ctg_ab_gmres(ctg_ctx *ctx, const ctg_geom *g, const float *b_dev,

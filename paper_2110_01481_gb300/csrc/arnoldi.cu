@@ -472,8 +472,12 @@ template <typename T, int E>
 __global__ void __launch_bounds__(kThreads, 2)
 gemv_kernel(const T *__restrict__ W, int64_t ldw, int k, const int *__restrict__ kdev, int koff,
             const double *__restrict__ y, const float *__restrict__ base, float *__restrict__ out,
-            int64_t L) {
+            int64_t L, const SolveIo *__restrict__ io) {
     extern __shared__ float s_y[];
+    if (io) {
+        base = io->x0;
+        out = io->x;
+    }
     if (kdev) k = *kdev + koff;
     for (int j = threadIdx.x; j < k; j += kThreads) s_y[j] = (float)y[j];
     __syncthreads();
@@ -490,9 +494,10 @@ gemv_kernel(const T *__restrict__ W, int64_t ldw, int k, const int *__restrict__
 // out = a - c (or a), res = ||out||^2; out may be the same vector as a or c.
 template <int E>
 __global__ void __launch_bounds__(kThreads, 2)
-sub_norm2_kernel(const float *a, const float *c, float *out, int64_t L,
+sub_norm2_kernel(const float *a, const float *const *a_at, const float *c, float *out, int64_t L,
                  float *__restrict__ partials,
                  unsigned *__restrict__ counter, double *__restrict__ res) {
+    if (a_at) a = *a_at;
     __shared__ float s_w[kWarps];
     const int tid = threadIdx.x;
     const int64_t g0 = (int64_t)blockIdx.x * kThreads * E + tid;
@@ -1166,7 +1171,7 @@ cudaError_t cgs2_loop_t(const T *W, int64_t ldw, int64_t L, float *q, const Loop
 
 template <typename T>
 cudaError_t gemv_t(const T *W, int64_t ldw, int64_t L, int k, const int *kdev, int koff, const double *y,
-                   const float *base, float *out, cudaStream_t st) {
+                   const float *base, float *out, cudaStream_t st, const SolveIo *io) {
     int E;
     const int G = ctg_red_grid(L, &E);
     const size_t smem = sizeof(float) * (size_t)(k > 0 ? k : 1);
@@ -1175,7 +1180,7 @@ cudaError_t gemv_t(const T *W, int64_t ldw, int64_t L, int k, const int *kdev, i
 #define CTG_GEMV_CASE(EE)                                                             \
     case EE:                                                                          \
         if ((err = ensure_smem(gemv_kernel<T, EE>, smem)) != cudaSuccess) return err; \
-        gemv_kernel<T, EE><<<G, kThreads, smem, st>>>(W, ldw, k, kdev, koff, y, base, out, L); \
+        gemv_kernel<T, EE><<<G, kThreads, smem, st>>>(W, ldw, k, kdev, koff, y, base, out, L, io); \
         break;
         CTG_GEMV_CASE(1)
         CTG_GEMV_CASE(2)
@@ -1247,25 +1252,26 @@ bool ctg_cgs2_fused_ok(int dtype, int64_t L, int kmax, const RedScratch &rs, boo
 int ctg_cgs2_fused_max(bool need_y) { return need_y ? kFusedMaxKY : kFusedMaxK; }
 
 cudaError_t ctg_gemv(const void *W, int dtype, int64_t ldw, int64_t L, int k, const double *y,
-                     const float *base, float *out, cudaStream_t st, const int *kdev, int koff) {
+                     const float *base, float *out, cudaStream_t st, const int *kdev, int koff,
+                     const SolveIo *io) {
     switch (dtype) {
-        case CTG_BASIS_FP32: return gemv_t(static_cast<const float *>(W), ldw, L, k, kdev, koff, y, base, out, st);
+        case CTG_BASIS_FP32: return gemv_t(static_cast<const float *>(W), ldw, L, k, kdev, koff, y, base, out, st, io);
         case CTG_BASIS_BF16:
-            return gemv_t(static_cast<const __nv_bfloat16 *>(W), ldw, L, k, kdev, koff, y, base, out, st);
+            return gemv_t(static_cast<const __nv_bfloat16 *>(W), ldw, L, k, kdev, koff, y, base, out, st, io);
         case CTG_BASIS_FP16:
-            return gemv_t(static_cast<const __half *>(W), ldw, L, k, kdev, koff, y, base, out, st);
+            return gemv_t(static_cast<const __half *>(W), ldw, L, k, kdev, koff, y, base, out, st, io);
         default: return cudaErrorInvalidValue;
     }
 }
 
 cudaError_t ctg_sub_norm2(const float *a, const float *c, float *out, int64_t L,
-                          double *res, const RedScratch &rs, cudaStream_t st) {
+                          double *res, const RedScratch &rs, cudaStream_t st, const float *const *a_at) {
     int E;
     const int G = ctg_red_grid(L, &E);
     switch (E) {
 #define CTG_SN_CASE(EE)                                                                        \
     case EE:                                                                                   \
-        sub_norm2_kernel<EE><<<G, kThreads, 0, st>>>(a, c, out, L, rs.partials, rs.counter, res); \
+        sub_norm2_kernel<EE><<<G, kThreads, 0, st>>>(a, a_at, c, out, L, rs.partials, rs.counter, res); \
         break;
         CTG_SN_CASE(1)
         CTG_SN_CASE(2)

@@ -490,7 +490,9 @@ constexpr int blk_tiles_y(int N, int nb) { return ((N + 1) / 2 + 16 * nb - 1) / 
 template <typename T, int kNB, int kSplit>
 __global__ void __cluster_dims__(1, 1, kSplit) __launch_bounds__(kBlkThreads, kNB == 4 ? 4 : 7)
 pixel_back_blocks_kernel(const T *__restrict__ b, ColRef bc, int N, int n_angles, int n_det,
-                         const BackAngle *__restrict__ tab, const float *__restrict__ add, float *__restrict__ x) {
+                         const BackAngle *__restrict__ tab, const float *__restrict__ add, float *__restrict__ x,
+                         const SolveIo *__restrict__ io) {
+    if (io) add = io->x0, x = io->x;
     pixel_back_blocks<T, kNB, kSplit>(b + col_offset(bc), N, n_angles, n_det, tab, add, x, blockIdx.x, blockIdx.y);
 }
 
@@ -500,7 +502,8 @@ template <typename T, int kModel, int kChunk, int kRows, int kSplit>
 __global__ void __cluster_dims__(1, 1, kSplit) __launch_bounds__(pair_threads<kRows>())
 pixel_pair_kernel(const T *__restrict__ b, ColRef bc, int N, int n_angles, int n_det,
                   const BackAngle *__restrict__ tab, int W, const MatchedAngle *__restrict__ mt, float thr,
-                  const float *__restrict__ add, float *__restrict__ x) {
+                  const float *__restrict__ add, float *__restrict__ x, const SolveIo *__restrict__ io) {
+    if (io) add = io->x0, x = io->x;
     pixel_pair_tile<T, kModel, kChunk, kRows, kSplit>(b + col_offset(bc), N, n_angles, n_det, tab, W, add, x,
                                                       blockIdx.x, blockIdx.y, mt, thr);
 }
@@ -513,8 +516,9 @@ template <typename T>
 __global__ void __launch_bounds__(kBX *kBY)
 pixel_back_kernel(const T *__restrict__ b, ColRef bc, int N, int n_angles, int n_det,
                   const BackAngle *__restrict__ tab, const float *__restrict__ add,
-                  float *__restrict__ x) {
+                  float *__restrict__ x, const SolveIo *__restrict__ io) {
     __shared__ float4 sp[kAChunk];
+    if (io) add = io->x0, x = io->x;
     b += col_offset(bc);
     const int j0 = blockIdx.x * kBX, i0 = blockIdx.y * kBY;
     const int dj = threadIdx.x, di = threadIdx.y;
@@ -612,6 +616,7 @@ template <typename T> struct BackArgs {
     const float *add;
     float *x;
     cudaStream_t st;
+    const SolveIo *io;
 };
 
 template <int kModel, int kChunk, int kRows, int kSplit, typename T>
@@ -619,14 +624,14 @@ void launch_pair(const BackArgs<T> &a) {
     const dim3 grid(back_tiles_x(a.N), back_tiles_y(a.N), kSplit);
     pixel_pair_kernel<T, kModel, kChunk, kRows, kSplit>
         <<<grid, pair_threads<kRows>(), pair_smem(kChunk, a.window), a.st>>>(
-            a.b, a.bc, a.N, a.n_angles, a.n_det, a.tab, a.window, a.mt, a.thr, a.add, a.x);
+            a.b, a.bc, a.N, a.n_angles, a.n_det, a.tab, a.window, a.mt, a.thr, a.add, a.x, a.io);
 }
 
 template <int kNB, int kSplit, typename T>
 void launch_blocks(const BackArgs<T> &a) {
     const dim3 grid(back_tiles_x(a.N), blk_tiles_y(a.N, kNB), kSplit);
     pixel_back_blocks_kernel<T, kNB, kSplit><<<grid, kBlkThreads, blk_smem(kNB), a.st>>>(
-        a.b, a.bc, a.N, a.n_angles, a.n_det, a.tab, a.add, a.x);
+        a.b, a.bc, a.N, a.n_angles, a.n_det, a.tab, a.add, a.x, a.io);
 }
 
 // blocks: the 2 x 2 block kernel (ctg_back_blocks_ok).  back_chunk: angles
@@ -653,7 +658,7 @@ cudaError_t launch_back_t(const BackArgs<T> &a, bool blocks, int back_chunk) {
     } else {
         dim3 grid((a.N + kBX - 1) / kBX, (a.N + kBY - 1) / kBY);
         pixel_back_kernel<T><<<grid, dim3(kBX, kBY), 0, a.st>>>(a.b, a.bc, a.N, a.n_angles, a.n_det, a.tab, a.add,
-                                                                a.x);
+                                                                a.x, a.io);
     }
     return cudaGetLastError();
 }
@@ -683,11 +688,11 @@ cudaError_t launch_matched_tiled_t(const BackArgs<T> &a) {
 cudaError_t ctg_launch_back_matched_tiled(const void *b, int dtype, int N, int n_angles, int n_det,
                                           const BackAngle *tab, int window, const MatchedAngle *mt,
                                           float thr, const float *add, float *x, cudaStream_t st,
-                                          ColRef bc) {
+                                          ColRef bc, const SolveIo *io) {
     if (window <= 0 || window > ctg_back_window_max()) return cudaErrorInvalidValue;
     auto run = [&](auto *p) {
         using T = typename std::remove_const<typename std::remove_pointer<decltype(p)>::type>::type;
-        return launch_matched_tiled_t(BackArgs<T>{p, bc, N, n_angles, n_det, tab, window, mt, thr, add, x, st});
+        return launch_matched_tiled_t(BackArgs<T>{p, bc, N, n_angles, n_det, tab, window, mt, thr, add, x, st, io});
     };
     switch (dtype) {
         case CTG_BASIS_FP32: return run(static_cast<const float *>(b));
@@ -699,10 +704,10 @@ cudaError_t ctg_launch_back_matched_tiled(const void *b, int dtype, int N, int n
 
 cudaError_t ctg_launch_back(const void *b, int dtype, int N, int n_angles, int n_det,
                             const BackAngle *tab, int window, bool blocks, const float *add, float *x,
-                            cudaStream_t st, int back_chunk, ColRef bc) {
+                            cudaStream_t st, int back_chunk, ColRef bc, const SolveIo *io) {
     auto run = [&](auto *p) {
         using T = typename std::remove_const<typename std::remove_pointer<decltype(p)>::type>::type;
-        return launch_back_t(BackArgs<T>{p, bc, N, n_angles, n_det, tab, window, nullptr, 0.0f, add, x, st}, blocks,
+        return launch_back_t(BackArgs<T>{p, bc, N, n_angles, n_det, tab, window, nullptr, 0.0f, add, x, st, io}, blocks,
                              back_chunk);
     };
     switch (dtype) {

@@ -105,16 +105,26 @@ __device__ __forceinline__ size_t col_offset(const ColRef &c) {
 }
 #endif
 
+// The caller's vectors of one GMRES solve, in its device state: kernels of a
+// captured solver loop read the pointers there when they run (arguments `at`
+// and `io` below; NULL: the pointer given), so that one captured loop serves
+// every set of vectors.
+struct SolveIo {
+    const float *b, *x0;   // x0: NULL for a zero start
+    float *x;
+    double target;         // tau ||e|| (0: no discrepancy stop)
+};
+
 // ---- projector launchers (projectors.cu, back.cu) --------------------------------
 // Stage x (n elements of type `dtype`, a CTG_BASIS_* value; column xc of a
 // basis at x when xc.k is set) for the forward projector.
 cudaError_t ctg_launch_pad(const void *x, int dtype, float2 *pad, int N, const PadLayout &pl,
-                           cudaStream_t st, ColRef xc = col_none());
+                           cudaStream_t st, ColRef xc = col_none(), const float *const *xat = nullptr);
 // Stage two images for ctg_launch_forward2, interleaved: x (type `dtype`,
 // column xc of a basis when xc.k is set) and x2 (FP32).  pad2 holds twice
 // the floats of pl (PadLayout::floats * 2).
 cudaError_t ctg_launch_pad2(const void *x, int dtype, ColRef xc, const float *x2, float4 *pad2, int N,
-                            const PadLayout &pl, cudaStream_t st);
+                            const PadLayout &pl, cudaStream_t st, float *const *x2at = nullptr);
 // Forward projector block shapes, the tile autotuner's candidates: angles
 // per block x angles per warp (a warp holds 32 / angles-per-warp adjacent
 // rays of each of its angles).  Every shape gives the same result bit for
@@ -177,7 +187,8 @@ bool ctg_back_blocks_ok(const BackAngle *host_tab, int n_angles);
 // bc: the input is column bc of a basis at b (bc.k set), or b itself.
 cudaError_t ctg_launch_back(const void *b, int dtype, int N, int n_angles, int n_det,
                             const BackAngle *tab, int window, bool blocks, const float *add, float *x,
-                            cudaStream_t st, int back_chunk = 32, ColRef bc = col_none());
+                            cudaStream_t st, int back_chunk = 32, ColRef bc = col_none(),
+                            const SolveIo *io = nullptr);     // io: add = io->x0, x = io->x
 
 // ---- matched back projector (matched.cu) ----------------------------------
 // x = B_thr b (+ add): the transpose of the forward projector, keeping the
@@ -185,13 +196,14 @@ cudaError_t ctg_launch_back(const void *b, int dtype, int N, int n_angles, int n
 // bins on each side beyond the two nearest (0 when ds >= max |c|).
 cudaError_t ctg_launch_back_matched(const void *b, int dtype, int N, int n_angles, int n_det,
                                     const BackAngle *tab, const MatchedAngle *mt, int rm, float thr,
-                                    const float *add, float *x, cudaStream_t st, ColRef bc = col_none());
+                                    const float *add, float *x, cudaStream_t st, ColRef bc = col_none(),
+                                    const SolveIo *io = nullptr);
 // The same with the tiled design of the pixel-driven B (back.cu), for
 // rm = 0 and window <= ctg_back_window_max().
 cudaError_t ctg_launch_back_matched_tiled(const void *b, int dtype, int N, int n_angles, int n_det,
                                           const BackAngle *tab, int window, const MatchedAngle *mt,
                                           float thr, const float *add, float *x, cudaStream_t st,
-                                          ColRef bc = col_none());
+                                          ColRef bc = col_none(), const SolveIo *io = nullptr);
 // *max_bits = bit pattern of max_ij A_ij (a float >= 0), on the device.
 cudaError_t ctg_matched_max(int N, int n_angles, int n_det, const BackAngle *tab,
                             const MatchedAngle *mt, int rm, unsigned *max_bits, cudaStream_t st);
@@ -282,10 +294,10 @@ int ctg_cgs2_fused_max(bool need_y);
 // that sizes the launch's shared memory).
 cudaError_t ctg_gemv(const void *W, int dtype, int64_t ldw, int64_t L, int k, const double *y,
                      const float *base, float *out, cudaStream_t st, const int *kdev = nullptr,
-                     int koff = 0);
+                     int koff = 0, const SolveIo *io = nullptr);     // io: base = io->x0, out = io->x
 // out = a - c (c may be NULL -> out = a) and *res = ||a - c||^2 (double, device).
 cudaError_t ctg_sub_norm2(const float *a, const float *c, float *out, int64_t L,
-                          double *res, const RedScratch &rs, cudaStream_t st);
+                          double *res, const RedScratch &rs, cudaStream_t st, const float *const *a_at = nullptr);
 // out = v / sqrt(*nrm2) rounded to `dtype` (nrm2 on device; out = 0 when
 // nrm2 == 0).
 cudaError_t ctg_scale(const float *v, const double *nrm2, void *out, int dtype, int64_t L,
@@ -297,6 +309,7 @@ enum { kRuleMaxit = 0, kRuleDP = 1, kRuleNCP = 2 };
 // Device state of one AB-/BA-GMRES solve.  The kernels of a step read k
 // here; the step's last kernel advances it or stops the solve.
 struct GmresState {
+    SolveIo io;           // written by the host before the solve's first kernel
     int k;                // the step being performed (1-based)
     int active;           // 1 while iterating
     int iters;            // k of the iterate to return
@@ -305,7 +318,6 @@ struct GmresState {
     int steps;            // steps executed
     int timed_out;        // a CGS2 grid barrier gave up
     int variant, rule, maxit;
-    double target;        // tau ||e||
     double beta;          // ||r0||
     double rho;           // |g_{k+1}| of the latest step (at exit: of the returned iterate)
     double resnorm;       // latest ||b - A x_k|| (BA with DP / NCP; at exit: of the returned iterate)
@@ -329,20 +341,21 @@ struct LoopBufs {
     double *scal;         // the reduction scratch's scalars
     double *h1;           // the reduction scratch's h1 (h1[k] = ||q_pre||^2)
     unsigned *counter;    // the reduction scratch's counters ([2]: barrier timeout)
-    cudaGraphConditionalHandle c_small, c_fused, c_pass;   // while-loop conditions (in_graph)
-    int in_graph;
+    cudaGraphConditionalHandle c_small, c_fused, c_pass;   // while-loop conditions of a captured solve
+    int loops;            // the loops with a condition (kLoopSmall | ..., 0: the host drives the steps)
     int small_max;        // last k of the loop of fused steps on one block per SM (0: none)
     int fused_max;        // last k of the fused-CGS2 loop
 };
+enum { kLoopSmall = 1, kLoopFused = 2, kLoopPass = 4 };
 // Modes of a step's Givens update: y_k every step (kGivY), AB NCP's
 // residual coefficients (kGivZ), the update ends the step (kGivEnd).
 enum { kGivY = 1, kGivZ = 2, kGivEnd = 4 };
-cudaError_t ctg_loop_init(const LoopBufs &B, int variant, int rule, int maxit, double target, cudaStream_t st);
+cudaError_t ctg_loop_init(const LoopBufs &B, int variant, int rule, int maxit, cudaStream_t st);
 // need_y: y_k every step; need_z: AB NCP residual coefficients; end: the
 // Givens kernel ends the step (AB with DP or maxit)
 cudaError_t ctg_loop_givens(const LoopBufs &B, bool need_y, bool need_z, bool end, int maxit, cudaStream_t st);
 // ||b - Ax||^2 (r_out: NULL or where b - Ax goes); decide: end the step (BA, DP)
-cudaError_t ctg_loop_resid(const LoopBufs &B, const float *b, const float *Ax, float *r_out, int64_t L,
+cudaError_t ctg_loop_resid(const LoopBufs &B, const float *Ax, float *r_out, int64_t L,
                            const RedScratch &rs, bool decide, cudaStream_t st);
 cudaError_t ctg_loop_ncp_decide(const LoopBufs &B, cudaStream_t st);
 cudaError_t ctg_loop_advance(const LoopBufs &B, cudaStream_t st);

@@ -28,10 +28,11 @@ __global__ void loop_givens_kernel(LoopBufs B, int mode, int pack_cap) {
 // pending maxit, else k + 1.  r_out: NULL, or where r is written (NCP).
 template <int E>
 __global__ void __launch_bounds__(kThreads, 2)
-loop_resid_kernel(const float *__restrict__ b, const float *__restrict__ Ax, float *__restrict__ r_out,
+loop_resid_kernel(const float *__restrict__ Ax, float *__restrict__ r_out,
                   int64_t L, float *__restrict__ partials, unsigned *__restrict__ counter, LoopBufs B,
                   int decide) {
     __shared__ float s_w[kWarps];
+    const float *b = B.S->io.b;
     const int tid = threadIdx.x;
     const int64_t g0 = (int64_t)blockIdx.x * kThreads * E + tid;
     float s = 0.f;
@@ -56,7 +57,7 @@ loop_resid_kernel(const float *__restrict__ b, const float *__restrict__ Ax, flo
     if (!decide) return;
     int stop = 0;
     if (S.pending == CTG_STOP_BREAKDOWN + 1) stop = S.pending;
-    else if (res <= S.target) stop = CTG_STOP_DP + 1;
+    else if (res <= S.io.target) stop = CTG_STOP_DP + 1;
     else stop = S.pending;
     S.pending = 0;
     end_step(B, stop, k);
@@ -92,14 +93,13 @@ __global__ void loop_advance_kernel(LoopBufs B) {
 // ||r0||^2 (AB: r0 = b - A x0; BA: r0 = B (b - A x0)), scal[4] =
 // ||b - A x0||^2 (BA), scal[6] = d_0 (NCP).  g = beta e1; a k = 0 stop when
 // beta = 0 (breakdown) or x0 already meets the discrepancy principle.
-__global__ void loop_init_kernel(LoopBufs B, int variant, int rule, int maxit, double target) {
+__global__ void loop_init_kernel(LoopBufs B, int variant, int rule, int maxit) {
     GmresState &S = *B.S;
     const double beta = sqrt(B.scal[2]);
     const double res0 = variant == CTG_BA ? sqrt(B.scal[4]) : beta;
     S.variant = variant;
     S.rule = rule;
     S.maxit = maxit;
-    S.target = target;
     S.beta = beta;
     S.res0 = res0;
     S.rho = beta;
@@ -117,13 +117,11 @@ __global__ void loop_init_kernel(LoopBufs B, int variant, int rule, int maxit, d
         S.dprev = B.scal[6];
         B.ncph[0] = B.scal[6];
     }
-    const bool dp0 = rule == kRuleDP && res0 <= target;
+    const bool dp0 = rule == kRuleDP && res0 <= S.io.target;
     if (dp0 || beta == 0.0) {
         S.active = 0;
         S.stop_reason = dp0 ? CTG_STOP_DP : CTG_STOP_BREAKDOWN;
-        set_cond(B.c_small, B.in_graph, 0u);
-        set_cond(B.c_fused, B.in_graph, 0u);
-        set_cond(B.c_pass, B.in_graph, 0u);
+        end_loops(B, kLoopSmall | kLoopFused | kLoopPass);
     } else {
         S.active = 1;
     }
@@ -163,8 +161,8 @@ int ensure_dyn_smem(const void *kern, size_t bytes) {
 int ctg_loop_pack_cap(int maxit) { return maxit < 160 ? maxit : 160; }
 static size_t pack_bytes(int cap) { return sizeof(double) * (size_t)cap * (cap + 1) / 2; }
 
-cudaError_t ctg_loop_init(const LoopBufs &B, int variant, int rule, int maxit, double target, cudaStream_t st) {
-    loop_init_kernel<<<1, 1, 0, st>>>(B, variant, rule, maxit, target);
+cudaError_t ctg_loop_init(const LoopBufs &B, int variant, int rule, int maxit, cudaStream_t st) {
+    loop_init_kernel<<<1, 1, 0, st>>>(B, variant, rule, maxit);
     return cudaGetLastError();
 }
 
@@ -177,14 +175,14 @@ cudaError_t ctg_loop_givens(const LoopBufs &B, bool need_y, bool need_z, bool en
     return cudaGetLastError();
 }
 
-cudaError_t ctg_loop_resid(const LoopBufs &B, const float *b, const float *Ax, float *r_out, int64_t L,
+cudaError_t ctg_loop_resid(const LoopBufs &B, const float *Ax, float *r_out, int64_t L,
                            const RedScratch &rs, bool decide, cudaStream_t st) {
     int E;
     const int G = ctg_red_grid(L, &E);
     switch (E) {
 #define CTG_LR_CASE(EE)                                                                                   \
     case EE:                                                                                              \
-        loop_resid_kernel<EE><<<G, kThreads, 0, st>>>(b, Ax, r_out, L, rs.partials, rs.counter, B, decide); \
+        loop_resid_kernel<EE><<<G, kThreads, 0, st>>>(Ax, r_out, L, rs.partials, rs.counter, B, decide); \
         break;
         CTG_LR_CASE(1)
         CTG_LR_CASE(2)

@@ -9,8 +9,11 @@
 
 namespace {
 
-__device__ __forceinline__ void set_cond(cudaGraphConditionalHandle h, bool in_graph, unsigned v) {
-    if (in_graph) cudaGraphSetConditional(h, v);
+__device__ __forceinline__ void end_loops(const LoopBufs &B, int which) {
+    const int w = which & B.loops;
+    if (w & kLoopSmall) cudaGraphSetConditional(B.c_small, 0u);
+    if (w & kLoopFused) cudaGraphSetConditional(B.c_fused, 0u);
+    if (w & kLoopPass) cudaGraphSetConditional(B.c_pass, 0u);
 }
 
 // End of step k (one thread): stop the solve with `stop` (a CTG_STOP_*
@@ -28,14 +31,12 @@ __device__ void end_step(const LoopBufs &B, int stop, int iters) {
         S.active = 0;
         S.stop_reason = stop - 1;
         S.iters = iters;
-        set_cond(B.c_small, B.in_graph, 0u);
-        set_cond(B.c_fused, B.in_graph, 0u);
-        set_cond(B.c_pass, B.in_graph, 0u);
+        end_loops(B, kLoopSmall | kLoopFused | kLoopPass);
     } else {
         const int k1 = S.k + 1;
         S.k = k1;
-        if (k1 > B.small_max) set_cond(B.c_small, B.in_graph, 0u);
-        if (k1 > B.fused_max) set_cond(B.c_fused, B.in_graph, 0u);
+        if (k1 > B.small_max) end_loops(B, kLoopSmall);
+        if (k1 > B.fused_max) end_loops(B, kLoopFused);
     }
 }
 
@@ -125,7 +126,7 @@ __device__ void loop_givens_warp(const LoopBufs &B, int k, const double *h, doub
     const int pending = brk ? CTG_STOP_BREAKDOWN + 1 : (k == S.maxit ? CTG_STOP_MAXIT + 1 : 0);
     if (mode & kGivEnd) {
         int stop = pending;
-        if (!brk && S.rule == kRuleDP && rho <= S.target) stop = CTG_STOP_DP + 1;
+        if (!brk && S.rule == kRuleDP && rho <= S.io.target) stop = CTG_STOP_DP + 1;
         end_step(B, stop, k);
     } else {
         S.pending = pending;

@@ -114,9 +114,14 @@ __device__ __forceinline__ void pad_pairs_block(const T *__restrict__ x, const f
 }
 
 // xc: the image is column xc of a basis (x + col_offset(xc)), or x itself.
+// at: the pointer of the FP32 image (x2 of two, else x) is read there.
 template <int kImgs, typename T>
 __global__ void pad_pairs_kernel(const T *__restrict__ x, ColRef xc, const float *__restrict__ x2,
-                                 void *__restrict__ pad, int N, int stride, int border) {
+                                 const float *const *at, void *__restrict__ pad, int N, int stride, int border) {
+    if (at) {
+        if constexpr (kImgs == 2) x2 = *at;
+        else if constexpr (std::is_same<T, float>::value) x = *at;
+    }
     pad_pairs_block<kImgs, T>(x + col_offset(xc), x2, pad, N, stride, border, blockIdx.x, blockIdx.y);
 }
 
@@ -617,19 +622,20 @@ int ctg_back_window(const BackAngle *host_tab, int n_angles) {
 }
 
 cudaError_t ctg_launch_pad(const void *x, int dtype, float2 *pad, int N, const PadLayout &pl,
-                           cudaStream_t st, ColRef xc) {
+                           cudaStream_t st, ColRef xc, const float *const *xat) {
+    if (xat && dtype != CTG_BASIS_FP32) return cudaErrorInvalidValue;
     dim3 grid((N + kPadTile - 1) / kPadTile, (N + kPadTile - 1) / kPadTile), block(kPadTile, kPadRows);
     switch (dtype) {
         case CTG_BASIS_FP32:
-            pad_pairs_kernel<1><<<grid, block, 0, st>>>(static_cast<const float *>(x), xc, nullptr, pad, N,
+            pad_pairs_kernel<1><<<grid, block, 0, st>>>(static_cast<const float *>(x), xc, nullptr, xat, pad, N,
                                                         pl.stride, pl.border);
             break;
         case CTG_BASIS_BF16:
             pad_pairs_kernel<1><<<grid, block, 0, st>>>(static_cast<const __nv_bfloat16 *>(x), xc, nullptr,
-                                                        pad, N, pl.stride, pl.border);
+                                                        nullptr, pad, N, pl.stride, pl.border);
             break;
         case CTG_BASIS_FP16:
-            pad_pairs_kernel<1><<<grid, block, 0, st>>>(static_cast<const __half *>(x), xc, nullptr, pad, N,
+            pad_pairs_kernel<1><<<grid, block, 0, st>>>(static_cast<const __half *>(x), xc, nullptr, nullptr, pad, N,
                                                         pl.stride, pl.border);
             break;
         default: return cudaErrorInvalidValue;
@@ -638,19 +644,20 @@ cudaError_t ctg_launch_pad(const void *x, int dtype, float2 *pad, int N, const P
 }
 
 cudaError_t ctg_launch_pad2(const void *x, int dtype, ColRef xc, const float *x2, float4 *pad2, int N,
-                            const PadLayout &pl, cudaStream_t st) {
+                            const PadLayout &pl, cudaStream_t st, float *const *x2at) {
+    const float *const *at = x2at;
     dim3 grid((N + kPadTile - 1) / kPadTile, (N + kPadTile - 1) / kPadTile), block(kPadTile, kPadRows);
     switch (dtype) {
         case CTG_BASIS_FP32:
-            pad_pairs_kernel<2><<<grid, block, 0, st>>>(static_cast<const float *>(x), xc, x2, pad2, N,
+            pad_pairs_kernel<2><<<grid, block, 0, st>>>(static_cast<const float *>(x), xc, x2, at, pad2, N,
                                                         pl.stride, pl.border);
             break;
         case CTG_BASIS_BF16:
-            pad_pairs_kernel<2><<<grid, block, 0, st>>>(static_cast<const __nv_bfloat16 *>(x), xc, x2, pad2,
-                                                        N, pl.stride, pl.border);
+            pad_pairs_kernel<2><<<grid, block, 0, st>>>(static_cast<const __nv_bfloat16 *>(x), xc, x2, at,
+                                                        pad2, N, pl.stride, pl.border);
             break;
         case CTG_BASIS_FP16:
-            pad_pairs_kernel<2><<<grid, block, 0, st>>>(static_cast<const __half *>(x), xc, x2, pad2, N,
+            pad_pairs_kernel<2><<<grid, block, 0, st>>>(static_cast<const __half *>(x), xc, x2, at, pad2, N,
                                                         pl.stride, pl.border);
             break;
         default: return cudaErrorInvalidValue;
