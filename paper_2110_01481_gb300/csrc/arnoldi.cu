@@ -4,7 +4,7 @@
 // (CGS2), which equals the paper's MGS loop in exact arithmetic but needs
 // three sweeps over W instead of k dependent ones:
 //   pass 1  h1 = W^T q,                ||q||^2      (one read of W)
-//   pass 2  q -= W h1,  h2 = W^T q,    ||q1||^2     (two reads of W)
+//   pass 2  q -= W h1,  h2 = W^T q,    ||q1||^2     (two reads of W, or one: cgs_sweep_kernel)
 //   pass 3  q -= W h2,  w_{k+1} = q / ||q||         (one read of W)
 // with ||q||^2 = ||q1||^2 - ||h2||^2 after pass 3 (exact for orthonormal W;
 // h2 is at the rounding level of ||q1|| after the first pass, so nothing
@@ -13,6 +13,7 @@
 // into per-block partials, and the last block to finish (atomic ticket, no
 // waiting) sums the partials in a fixed order (compensated FP32 pairs,
 // FP64 results), so results are deterministic run to run.
+#include <algorithm>
 #include <atomic>
 
 #include "loop_device.cuh"
@@ -182,6 +183,151 @@ cgs_pass_kernel(const T *__restrict__ W, int64_t ldw, int k, const int *__restri
     if (kdev) k = *kdev;
     cgs_pass_body<T, E, UPDATE, DOTS, NORM>(W, ldw, k, q, L, coef, partials, counter, red_out,
                                             blockIdx.x, gridDim.x);
+}
+
+// The second pass for a large FP32 basis: q -= W coef, then red_out = [W^T q,
+// q^T q], with one read of W (cgs_pass_kernel's two loops over the vectors
+// read its slice twice, from memory both times once the slices of the resident
+// blocks are more than L2 holds).  Streams of kNW warps, eight warps to a
+// block and one block to an SM, walk over groups of 128 columns; warp w of a
+// stream holds W_j of the group for the vectors j = w, w + kNW, ..., four
+// columns per lane, in registers: its part of W coef goes through shared
+// memory (one barrier of the stream per group), and the new q of its lanes'
+// columns meets the same registers for the dots, whose partial sums stay with
+// the lane until the last group.  Each thread's loads run ahead through a ring
+// of `depth` groups in shared memory (cp.async of its own 16 bytes per vector,
+// read by itself alone); a slot is refilled after the barrier that follows its
+// last read.  The last warp, which never has more vectors than the others,
+// also carries q.  Memory bounds it: 5.9 TB/s at L = 4.19M, k = 60, 277 us
+// with two reads and 172 us with one; 76 to 53 us at k = 16; 320 to 174 us at
+// L = 1.25M, k = 200; 117 to 74 us at L = 1M, k = 100.  What is missing to the
+// copy's 6.8 TB/s are SMs that get less bandwidth than others and finish last
+// (a fifth of the SM time at the end); holding the others back made it slower.
+constexpr int kSweepCols = 128;
+constexpr int kSweepMaxDepth = 4;
+
+__device__ __forceinline__ void cp_async16(float4 *dst, const float *src, int bytes) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// waits until at most depth - 1 of the thread's groups are in flight
+__device__ __forceinline__ void cp_wait_oldest(int depth) {
+    switch (depth) {
+        case 1: asm volatile("cp.async.wait_group 0;" ::: "memory"); break;
+        case 2: asm volatile("cp.async.wait_group 1;" ::: "memory"); break;
+        case 3: asm volatile("cp.async.wait_group 2;" ::: "memory"); break;
+        default: asm volatile("cp.async.wait_group 3;" ::: "memory"); break;
+    }
+}
+
+// bytes of shared memory: the rings (k + 1 rows of 512 bytes per group),
+// the two exchange buffers, the coefficients
+__host__ __device__ constexpr size_t sweep_smem(int k, int depth, int streams) {
+    return 512 * ((size_t)streams * depth * (k + 1) + 2 * kWarps) + sizeof(float) * (size_t)k;
+}
+
+template <int NJ, int kNW>
+__global__ void __launch_bounds__(kThreads, 1)
+cgs_sweep_kernel(const float *__restrict__ W, int64_t ldw, int k, int depth,
+                 float *__restrict__ q, int64_t L, const double *__restrict__ coef, float *__restrict__ partials,
+                 unsigned *__restrict__ counter, double *__restrict__ red_out) {
+    extern __shared__ float4 smem4[];
+    constexpr int kStreams = kWarps / kNW;
+    const int tid = threadIdx.x, lane = tid & 31, stream = (tid >> 5) / kNW, warp = (tid >> 5) % kNW;
+    const int stage = (k + 1) * 32;                          // float4s per group in a ring
+    float4 *ringq = smem4 + stream * depth * stage + k * 32 + lane;
+    float4 *ring = ringq - k * 32 + warp * 32;               // vector warp + kNW jj: + 32 kNW jj
+    float4 *xch = smem4 + kStreams * depth * stage;          // [2][kWarps][32]
+    float *s_coef = reinterpret_cast<float *>(xch + 2 * kWarps * 32);
+    const bool has_q = warp == kNW - 1;
+    for (int j = tid; j < k; j += kThreads) s_coef[j] = (float)coef[j];
+    const int64_t ngroups = (L + kSweepCols - 1) / kSweepCols;
+    // from the last columns to the first: the pass before read the last ones last
+    const int first = blockIdx.x * kStreams + stream, step = gridDim.x * kStreams;
+    int64_t next = ngroups - 1 - first;
+    const float *W0 = W + (int64_t)warp * ldw;
+    auto fetch = [&](int slot) {
+        if (next >= 0) {
+            const int64_t c = next * kSweepCols + 4 * lane;
+            const int bytes = c + 4 <= L ? 16 : (c < L ? 4 * (int)(L - c) : 0);
+            const int64_t at = bytes ? c : 0;
+            const float *src = W0 + at;
+            float4 *dst = ring + slot * stage;
+#pragma unroll
+            for (int jj = 0; jj < NJ; ++jj)
+                if (warp + kNW * jj < k) cp_async16(dst + 32 * kNW * jj, src + (int64_t)(kNW * jj) * ldw, bytes);
+            if (has_q) cp_async16(ringq + slot * stage, q + at, bytes);
+        }
+        cp_commit();
+        next -= step;
+    };
+    for (int s = 0; s < depth; ++s) fetch(s);
+    float acc[NJ], nrm = 0.f;
+#pragma unroll
+    for (int jj = 0; jj < NJ; ++jj) acc[jj] = 0.f;
+    __syncthreads();                                         // the coefficients
+    int slot = 0, buf = 0;
+    for (int64_t grp = ngroups - 1 - first; grp >= 0; grp -= step) {
+        cp_wait_oldest(depth);
+        float4 w[NJ];
+        const float4 *src = ring + slot * stage;
+#pragma unroll
+        for (int jj = 0; jj < NJ; ++jj)
+            if (warp + kNW * jj < k) w[jj] = src[32 * kNW * jj];
+        float4 p = has_q ? ringq[slot * stage] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int jj = 0; jj < NJ; ++jj)
+            if (warp + kNW * jj < k) {
+                const float c = s_coef[warp + kNW * jj];
+                p.x = fmaf(-c, w[jj].x, p.x);
+                p.y = fmaf(-c, w[jj].y, p.y);
+                p.z = fmaf(-c, w[jj].z, p.z);
+                p.w = fmaf(-c, w[jj].w, p.w);
+            }
+        float4 *x = xch + (buf * kWarps + stream * kNW) * 32 + lane;
+        if (kNW > 1) {
+            x[warp * 32] = p;
+            asm volatile("bar.sync %0, %1;" ::"r"(stream + 1), "n"(32 * kNW) : "memory");
+        } else {
+            __syncwarp();
+        }
+        fetch(slot);
+        float4 v = kNW > 1 ? x[0] : p;
+#pragma unroll
+        for (int u = 1; u < kNW; ++u) {
+            const float4 t = x[u * 32];
+            v.x += t.x;
+            v.y += t.y;
+            v.z += t.z;
+            v.w += t.w;
+        }
+#pragma unroll
+        for (int jj = 0; jj < NJ; ++jj)
+            if (warp + kNW * jj < k) acc[jj] += dot4(w[jj], v);
+        if (has_q) {
+            st4(q, grp * (kSweepCols / 4) + lane, L, v);
+            nrm += dot4(v, v);
+        }
+        buf ^= 1;
+        if (++slot == depth) slot = 0;
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    // the lanes' sums in the layout of block_reduce_finish (a row per warp,
+    // zero where the vector is another warp's), over the ring
+    float *s_w = reinterpret_cast<float *>(smem4);
+    const int nred = k + 1;
+    for (int j = tid; j < kWarps * nred; j += kThreads) s_w[j] = 0.f;
+    __syncthreads();
+#pragma unroll
+    for (int jj = 0; jj < NJ; ++jj) {
+        const float t = warp_sum(acc[jj]);
+        if (lane == 0 && warp + kNW * jj < k) s_w[(tid >> 5) * nred + warp + kNW * jj] = t;
+    }
+    nrm = warp_sum(nrm);
+    if (lane == 0 && has_q) s_w[(tid >> 5) * nred + k] = nrm;
+    block_reduce_finish(s_w, nred, partials, counter, red_out, blockIdx.x, gridDim.x);
 }
 
 // Every block sums the partial rows [row0, row0 + nrows) of all blocks in
@@ -1113,13 +1259,65 @@ cudaError_t fused_dispatch(const T *W, int64_t ldw, int64_t L, int k, float *q, 
     }
 }
 
+// Up to kSweepMaxK vectors the one-read second pass (cgs_sweep_kernel) serves
+// an FP32 basis of 100 MB or more (with kSweepMinK vectors: below, its groups
+// are too small for what a group costs), and any basis of more than kFusedMaxK
+// vectors, whose short slices cgs_pass_kernel spreads over few blocks.  Its
+// time against cgs_pass_kernel's two reads (us): L = 2.4M, k = 12 (115 MB)
+// 26 / 30; 522,000 x 60 (125 MB) 27 / 31; 522,000 x 40 (84 MB) 23 / 21;
+// 4.19M x 8 36 / 40 and x 4 34 / 20; 131,072 x 150 28 / 34; 4,099 x 200 16 / 42.
+constexpr int kSweepMinK = 8, kSweepMaxK = 216;
+constexpr int64_t kSweepMinBytes = 100000000;
+// From 300 MB on, the passes with it are faster than the one-launch step with
+// its re-reads of W: 221 / 233 us at L = 2.4M, k = 40, 228 / 275 us at 1M x
+// 100, level at 522,000 x 90 (188 MB).
+constexpr int64_t kSweepNotFusedBytes = 300000000;
+
+template <typename T>
+bool sweep_serves(int64_t L, int k, int64_t min_bytes) {
+    return std::is_same<T, float>::value && k >= kSweepMinK && k <= kSweepMaxK && 4 * L * k >= min_bytes;
+}
+
+template <int NJ, int kNW>
+cudaError_t launch_sweep(const float *W, int64_t ldw, int k, float *q, int64_t L, const RedScratch &rs,
+                         cudaStream_t st) {
+    constexpr int streams = kWarps / kNW;
+    static_assert(sweep_smem(NJ * kNW <= kSweepMaxK ? NJ * kNW : kSweepMaxK, 1, streams) <= 226 * 1024, "ring");
+    int depth = kSweepMaxDepth;
+    while (depth > 1 && sweep_smem(k, depth, streams) > 226 * 1024) --depth;
+    const size_t smem = sweep_smem(k, depth, streams);
+    const cudaError_t err = ensure_smem(cgs_sweep_kernel<NJ, kNW>, smem);
+    if (err != cudaSuccess) return err;
+    const int64_t groups = (L + kSweepCols - 1) / kSweepCols;
+    const int G = (int)std::min<int64_t>((groups + streams - 1) / streams, ctg_target_grid() / 2);
+    cgs_sweep_kernel<NJ, kNW><<<G, kThreads, smem, st>>>(W, ldw, k, depth, q, L, rs.h1, rs.partials, rs.counter,
+                                                         rs.h2);
+    return cudaGetLastError();
+}
+
+// Pass 2: q -= W h1, h2 = [W^T q, ||q||^2].  Fewer warps to a stream exchange
+// less, but hold more vectors each.
+template <typename T>
+cudaError_t second_pass(const T *W, int64_t ldw, int k, float *q, int64_t L, const RedScratch &rs, cudaStream_t st) {
+    if constexpr (std::is_same<T, float>::value) {
+        if (sweep_serves<T>(L, k, k > kFusedMaxK ? 0 : kSweepMinBytes)) {
+            if (k <= 16) return launch_sweep<16, 1>(W, ldw, k, q, L, rs, st);
+            if (k <= 32) return launch_sweep<16, 2>(W, ldw, k, q, L, rs, st);
+            if (k <= 64) return launch_sweep<16, 4>(W, ldw, k, q, L, rs, st);
+            if (k <= 128) return launch_sweep<32, 4>(W, ldw, k, q, L, rs, st);
+            return launch_sweep<27, 8>(W, ldw, k, q, L, rs, st);
+        }
+    }
+    return launch_pass<T, true, true, true>(W, ldw, k, nullptr, q, L, rs.h1, rs, rs.h2, st);
+}
+
 template <typename T>
 cudaError_t cgs2_step_t(const T *W, int64_t ldw, int64_t L, int k, float *q, T *w_out,
                         double *h_out, const RedScratch &rs, long long spin_limit, cudaStream_t st,
                         int *nkern) {
     cudaError_t err;
     if (nkern) *nkern = k > 0 ? 3 : 2;
-    if (k <= kFusedMaxK && rs.rows >= 2 * k + 2) {
+    if (k <= kFusedMaxK && rs.rows >= 2 * k + 2 && !sweep_serves<T>(L, k, kSweepNotFusedBytes)) {
         bool done = false;
         err = fused_dispatch<T>(W, ldw, L, k, q, w_out, h_out, nullptr, rs, spin_limit, true, st, &done);
         if (err != cudaSuccess) return err;
@@ -1135,7 +1333,7 @@ cudaError_t cgs2_step_t(const T *W, int64_t ldw, int64_t L, int k, float *q, T *
         return err;
     if (k > 0) {
         // pass 2: q -= W h1; h2 = W^T q, ||q||^2 (h2[k])
-        if ((err = launch_pass<T, true, true, true>(W, ldw, k, nullptr, q, L, rs.h1, rs, rs.h2, st)) != cudaSuccess)
+        if ((err = second_pass<T>(W, ldw, k, q, L, rs, st)) != cudaSuccess)
             return err;
         // q -= W h2 and w_out = q / ||q|| in one sweep; ||q||^2 -> scal[1]
         return launch_update_scale<T>(W, ldw, k, nullptr, nullptr, 0, q, L, rs, w_out, h_out, st);
