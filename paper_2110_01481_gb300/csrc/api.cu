@@ -509,13 +509,13 @@ int get_geom(ctg_ctx *ctx, const ctg_geom *g, GeomEntry **out) {
         err = cudaMemcpy(e.back, bk.data(), sizeof(BackAngle) * bk.size(), cudaMemcpyHostToDevice);
     if (err == cudaSuccess) {
         std::vector<int> orders[kFwdShapes + 1], all;
-        std::vector<int2> ranges;
+        const std::vector<int2> ranges = ctg_forward_ranges(fw.data(), g->N, g->n_angles, g->n_det);
         ctg_forward_plan(fw.data(), g->N, g->n_angles, g->n_det, e.pl, 1, e.fwd_groups,
-                         {kFwdShapeWarps[0], kFwdShapeWarps[1]}, orders);
+                         {kFwdShapeWarps[0], kFwdShapeWarps[1]}, orders, ranges);
         ctg_forward_plan(fw.data(), g->N, g->n_angles, g->n_det, e.pl, 4, e.fwd_groups,
-                         {kFwdShapeWarps[2], kFwdShapeWarps[3]}, orders + 2, &ranges);
+                         {kFwdShapeWarps[2], kFwdShapeWarps[3]}, orders + 2, ranges);
         ctg_forward_plan(fw.data(), g->N, g->n_angles, g->n_det, e.pl, 8, e.fwd_groups,
-                         {kFwdShapeWarps[kFwdShapeTwo]}, orders + kFwdShapeTwo, &ranges);
+                         {kFwdShapeWarps[kFwdShapeTwo]}, orders + kFwdShapeTwo, ranges);
         for (int c = 0; c <= kFwdShapes; ++c) {
             e.fwd_order_off[c] = all.size();
             all.insert(all.end(), orders[c].begin(), orders[c].end());

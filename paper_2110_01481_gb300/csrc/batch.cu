@@ -52,10 +52,10 @@ std::shared_ptr<const FwdPlan> plan_forward(const ctg_geom &g, std::vector<FwdAn
     auto f = std::make_shared<FwdPlan>();
     const PadLayout pl = ctg_pad_layout(g.N, g.det_spacing);
     f->groups = ctg_forward_groups(fw);
-    std::vector<int2> ranges;
+    const std::vector<int2> ranges = ctg_forward_ranges(fw.data(), g.N, g.n_angles, g.n_det);
     for (const int split : {1, 4, 8})
         ctg_forward_plan(fw.data(), g.N, g.n_angles, g.n_det, pl, split, f->groups, {kBatchFwdWarps},
-                         &f->order[fwd_split_index(split)], &ranges);
+                         &f->order[fwd_split_index(split)], ranges);
     return f;
 }
 

@@ -168,11 +168,12 @@ int ctg_fwd_blocks(int warps, int split, int ngroups, int n_det);
 // blocks (tile index by * gx + bx, bx the ray group and by the block's place
 // among the angle groups): longest estimated walk first, which shortens the
 // tail of the launch where the chord lengths, and so the blocks' run times,
-// differ.  From the host copy of the angle table.  ranges: filled by split 4
-// (the walks' row ranges) and read by split 8, which comes after it.
+// differ.  From the host copy of the angle table and its walks' ranges
+// (ctg_forward_ranges), which serve every split.
+std::vector<int2> ctg_forward_ranges(const FwdAngle *host_tab, int N, int n_angles, int n_det);
 void ctg_forward_plan(const FwdAngle *host_tab, int N, int n_angles, int n_det, const PadLayout &pl, int split,
                       FwdGroups &G, std::initializer_list<int> warps, std::vector<int> *orders,
-                      std::vector<int2> *ranges = nullptr);
+                      const std::vector<int2> &ranges);
 // Detector-window width (in bins) that the tiled back projector stages per
 // angle, from the host copy of the angle table.
 int ctg_back_window(const BackAngle *host_tab, int n_angles);

@@ -798,40 +798,40 @@ void longest_first(const std::vector<int> &cost, int ng, int gx, int W, std::vec
 }
 }  // namespace
 
+// Row ranges [x, y] of the walks of each angle's groups of eight rays.
+std::vector<int2> ctg_forward_ranges(const FwdAngle *tab, int N, int n_angles, int n_det) {
+    const int gx = (n_det + 7) / 8;
+    std::vector<int2> r((size_t)n_angles * gx);
+    for (int a = 0; a < n_angles; ++a)
+        for (int bx = 0; bx < gx; ++bx) {
+            int2 &w = r[(size_t)a * gx + bx];
+            group_range(tab[a], N, 8 * bx, std::min(n_det, 8 * bx + 8), w.x, w.y);
+        }
+    return r;
+}
+
 void ctg_forward_plan(const FwdAngle *tab, int N, int n_angles, int n_det, const PadLayout &pl, int split,
                       FwdGroups &G, std::initializer_list<int> warps, std::vector<int> *orders,
-                      std::vector<int2> *ranges) {
+                      const std::vector<int2> &ranges) {
     const int R = 32 / split, gx = (n_det + R - 1) / R, ng = G.count[fwd_split_index(split)];
     // groups cut short by changes of drive leave lanes idle: not worth it when
     // more than a fifth are (widely spaced angles)
     bool safe = split == 1 || (long long)ng * split * 4 <= 5LL * n_angles + 12 * split;
-    // eight angles and four rays: from the ranges of the two groups of four
-    // (each group of eight is one or two of them) and their eight rays
-    const int gx4 = (n_det + 7) / 8;
-    if (split == 4) ranges->resize((size_t)ng * gx);
+    const int gx8 = (n_det + 7) / 8;      // the ranges' groups of eight rays
     // steps of each warp's lockstep walk plus a fixed cost
     std::vector<int> cost((size_t)ng * gx);
-    for (int g = 0, g4 = 0; g < ng; ++g) {
+    for (int g = 0; g < ng; ++g) {
         const unsigned w = split == 8 ? tab[g].row_group8 : tab[g].group4;
         const int a0 = split == 1 ? g : (int)(w >> 4), na = split == 1 ? 1 : (int)((w >> 1) & 7u) + 1;
         for (int bx = 0; bx < gx; ++bx) {
             const int d0 = bx * R, d1 = std::min(n_det, d0 + R);
             int wlo = N, whi = -1;
-            if (split == 8) {
-                for (int h = 0; h < (na > 4 ? 2 : 1); ++h) {
-                    const int2 r = (*ranges)[(size_t)(g4 + h) * gx4 + bx / 2];
+            for (int a = a0; a < a0 + na; ++a)
+                for (int r8 = d0 / 8; 8 * r8 < d1; ++r8) {
+                    const int2 r = ranges[(size_t)a * gx8 + r8];
                     wlo = std::min(wlo, r.x);
                     whi = std::max(whi, r.y);
                 }
-            } else {
-                for (int a = a0; a < a0 + na; ++a) {
-                    int lo, hi;
-                    group_range(tab[a], N, d0, d1, lo, hi);
-                    wlo = std::min(wlo, lo);
-                    whi = std::max(whi, hi);
-                }
-                if (split == 4) (*ranges)[(size_t)g * gx + bx] = make_int2(wlo, whi);
-            }
             cost[(size_t)g * gx + bx] = (whi >= wlo ? whi - (wlo & ~3) + 1 : 0) + 16;
             if (!safe || split == 1 || pl.clamp || whi < wlo) continue;     // clamped indices are safe
             // the device's range may differ from this estimate by a step:
@@ -848,7 +848,6 @@ void ctg_forward_plan(const FwdAngle *tab, int N, int n_angles, int n_det, const
             }
             if ((least >> CTG_FXF_BITS) < -pl.border || (most >> CTG_FXF_BITS) > N - 1 + pl.border) safe = false;
         }
-        g4 += na > 4 ? 2 : 1;
     }
     G.safe[fwd_split_index(split)] = safe;
     for (const int W : warps) longest_first(cost, ng, gx, W, *orders++);
