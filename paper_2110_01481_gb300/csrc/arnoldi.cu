@@ -351,7 +351,7 @@ __device__ __forceinline__ void write_rows(const float *s_w, int nred, int row0,
 // with a bounded wait: thread 0 of each block adds one arrival to *count
 // and waits until `target` arrivals are in (target = barrier index x grid
 // size, so one counter serves successive barriers).  After spin_limit polls
-// (about 100 ns apart) it gives up: it sets *err and returns false, as does
+// (some 400 ns apart) it gives up: it sets *err and returns false, as does
 // every block that finds *err set while it waits, so no block waits for
 // ever.  Returns true when the barrier completed.
 __device__ __forceinline__ bool grid_barrier(unsigned *count, unsigned target, long long spin_limit,
@@ -359,8 +359,9 @@ __device__ __forceinline__ bool grid_barrier(unsigned *count, unsigned target, l
     __shared__ int s_ok;
     __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(count, 1u);
+        // release: the block's writes before the barrier above; the acquiring
+        // load and the barrier below give the block the others' writes
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
         int ok = 1;
         long long spins = 0;
         for (;;) {
@@ -374,9 +375,8 @@ __device__ __forceinline__ bool grid_barrier(unsigned *count, unsigned target, l
                 ok = 0;
                 break;
             }
-            __nanosleep(100);
+            __nanosleep(32);
         }
-        __threadfence();
         s_ok = ok;
     }
     __syncthreads();
@@ -401,10 +401,10 @@ __device__ __forceinline__ bool grid_barrier(unsigned *count, unsigned target, l
 // the last block to leave sets it back to zero); on a timeout h_out[0..k]
 // is set to NaN.
 // With giv_mode >= 0 (a step of the device-driven solver loop), block 0
-// then runs the step's FP64 Givens update (loop_givens_warp) on the column it
-// has just written, and, by the mode, the end of the step, so the step needs
-// no launch of its own for them; its shared memory holds kcap_giv staging
-// entries and the packed triangle for y_k beyond the step's own.
+// then runs the step's FP64 Givens update (loop_givens_staged) on the column it
+// has just formed, and, by the mode, the end of the step, so the step needs
+// no launch of its own for them; its shared memory holds the update's stage
+// for k <= kcap_giv and the packed triangle for y_k beyond the step's own.
 template <typename T, int E>
 __global__ void __launch_bounds__(kThreads, 2)
 cgs2_fused_kernel(const T *__restrict__ W, int64_t ldw, int k, const int *__restrict__ kdev,
@@ -413,14 +413,15 @@ cgs2_fused_kernel(const T *__restrict__ W, int64_t ldw, int k, const int *__rest
                   double *__restrict__ h1g, double *__restrict__ h2g, double *__restrict__ scal,
                   unsigned *__restrict__ bar, int *__restrict__ err, long long spin_limit,
                   LoopBufs lb, int giv_mode, int kcap_giv, int pack_cap) {
+    // with giv_mode >= 0 k <= kcap_giv, at most 128 and with kGivY 64 (launch_fused)
     if (kdev) {
         k = *kdev;
         w_out = const_cast<T *>(W) + (size_t)k * ldw;
         h_out = H + (size_t)(k - 1) * ldh;
     }
     extern __shared__ double smem_d[];
-    double *s_stage = smem_d;                       // 3 kcap_giv + 1: the Givens staging
-    double *s_pack = s_stage + (giv_mode >= 0 ? 3 * kcap_giv + 1 : 0);   // packed R for y_k
+    double *s_stage = smem_d;                       // the Givens update's stage
+    double *s_pack = s_stage + (giv_mode >= 0 ? givens_stage_doubles(kcap_giv) : 0);   // packed R for y_k
     double *s_h1 = s_pack + (giv_mode >= 0 && (giv_mode & kGivY) ? pack_cap * (pack_cap + 1) / 2 : 0);
     double *s_h2 = s_h1 + (k + 1);                  // k + 2: h2, ||q1||^2, then ||q2||^2
     float *s_c = reinterpret_cast<float *>(s_h2 + (k + 2));   // k coefficients
@@ -431,8 +432,12 @@ cgs2_fused_kernel(const T *__restrict__ W, int64_t ldw, int k, const int *__rest
     float4 qv[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) qv[e] = ld4_rw(q, g0 + (int64_t)e * kThreads, L);
+    const bool givens = giv_mode >= 0 && blk == 0;
+    const GivensStage stage = givens_stage(s_stage, kcap_giv, s_pack);
+    if (givens) givens_fetch(lb, k, giv_mode, stage);
     // pass 1: h1 = W^T q, ||q||^2
     dots_slice<T, E, true, true>(W, ldw, k, g0, L, qv, s_w, k + 1);
+    if (givens) asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     write_rows(s_w, k + 1, 0, partials, Gp, blk);
     bool ok = grid_barrier(bar, (unsigned)G, spin_limit, err);
@@ -477,10 +482,10 @@ cgs2_fused_kernel(const T *__restrict__ W, int64_t ldw, int k, const int *__rest
         // Givens update takes the NaN column for a breakdown, and the step's
         // end reports the timeout
         for (int j = tid; j <= k; j += kThreads) h_out[j] = __longlong_as_double(0x7ff8000000000000LL);
-        if (giv_mode >= 0 && blk == 0) {
-            __syncthreads();
-            if (tid < 32) loop_givens_warp(lb, k, h_out, 0.0, giv_mode, s_pack, pack_cap,
-                                           k <= kcap_giv ? s_stage : nullptr);
+        if (givens && tid < 32) {
+            for (int j = tid; j <= k; j += 32) stage.h[j] = __longlong_as_double(0x7ff8000000000000LL);
+            __syncwarp();
+            loop_givens_staged(lb, k, 0.0, giv_mode, stage);
         }
         return;
     }
@@ -510,11 +515,13 @@ cgs2_fused_kernel(const T *__restrict__ W, int64_t ldw, int k, const int *__rest
     }
     // the last block out resets the barrier counter for the next launch
     // (every block has read k by now: it passed both barriers)
-    if (tid == 0 && atomicAdd(bar, 1u) == (nbar + 1u) * (unsigned)G - 1u) atomicExch(bar, 0u);
-    if (giv_mode >= 0 && blk == 0) {
-        __syncthreads();                            // the column is written
-        if (tid < 32) loop_givens_warp(lb, k, h_out, s_h1[k], giv_mode, s_pack, pack_cap,
-                                       k <= kcap_giv ? s_stage : nullptr);
+    // (not by the warp of the Givens update, which would wait for the answer)
+    if (tid == 32 && atomicAdd(bar, 1u) == (nbar + 1u) * (unsigned)G - 1u) atomicExch(bar, 0u);
+    if (givens && tid < 32) {
+        for (int j = tid; j < k; j += 32) stage.h[j] = s_h1[j] + s_h2[j];
+        if (tid == 0) stage.h[k] = nrm2 * rnorm;
+        __syncwarp();
+        loop_givens_staged(lb, k, s_h1[k], giv_mode, stage);
     }
 }
 
@@ -1144,12 +1151,12 @@ void ctg_red_scratch_carve(void *base, int64_t L, int kmax, RedScratch *rs) {
 
 namespace {
 
-// giv_mode >= 0: with the Givens staging (3 k + 1 doubles) and, for y_k,
+// giv_mode >= 0: with the Givens update's stage and, for y_k,
 // the packed triangle (loop_pack_cap(k) columns) in front
 size_t fused_smem_bytes(int k, int giv_mode = -1) {
     size_t giv = 0;
     if (giv_mode >= 0) {
-        giv = 3 * (size_t)k + 1;
+        giv = givens_stage_doubles(k);
         if (giv_mode & kGivY) giv += (size_t)loop_pack_cap(k) * (loop_pack_cap(k) + 1) / 2;
     }
     return sizeof(double) * (giv + 2 * (size_t)k + 3) + sizeof(float) * ((size_t)k + (size_t)kWarps * (k + 1));
