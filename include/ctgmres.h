@@ -164,7 +164,8 @@ int ctg_backproject(ctg_ctx *ctx, const ctg_geom *g, const float *b_dev,
  * per warp, 8 adjacent rays of each), and the pixel-driven back projector
  * with 16, 32 and 64 angles staged per pass (CUDA events, 3 launches each on
  * zero inputs, with temporary buffers of about 5n + m floats), and keeps the
- * fastest.  The shapes with 4 angles per warp are candidates only where the
+ * fastest (at a pitch of a pixel or more the back projector has one form,
+ * timed once).  The shapes with 4 angles per warp are candidates only where the
  * host has checked that every warp's walk stays inside the staged image
  * (adjacent angles of a fine angular sampling; not widely spaced ones).  The
  * candidates sum every ray and every pixel in the same order, so results do

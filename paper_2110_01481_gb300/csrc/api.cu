@@ -407,12 +407,17 @@ int tune_geometry(GeomEntry *ge) {
     }
     const int back_cand[3] = {16, 32, 64};
     if (g->back_model == CTG_BACK_PIXEL)
-        for (int c = 0; c < 3; ++c)
+        for (int c = 0; c < 3; ++c) {
+            if (c > 0 && ge->back_blocks) {         // its kernel has no pass size: one time for all three
+                ge->back_us[c] = ge->back_us[0];
+                continue;
+            }
             timed([&] {
                 if (err == cudaSuccess)
                     err = ctg_launch_back(bv, CTG_BASIS_FP32, g->N, g->n_angles, g->n_det, ge->back,
                                           ge->back_window, ge->back_blocks, nullptr, xv, st, back_cand[c]);
             }, &ge->back_us[c]);
+        }
     if (err == cudaSuccess) {
         int fs = 0;
         for (int c = 1; c < kFwdShapes; ++c)
