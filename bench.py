@@ -857,7 +857,7 @@ def run_gpu(args):
             kname = "joseph_forward_kernel"
         else:
             interp = n * N_ANG
-            kname = "pixel_back_tiled_kernel"
+            kname = "pixel_back_blocks_kernel"
         per_launch_s = phases[dom]["ms"] / 1e3 / phases[dom]["calls"]
         ach = 8.0 * interp / per_launch_s / 1e9
         l1, sms, mhz = l1_peak(torch, dev, clocks.get("sm_max_mhz"))

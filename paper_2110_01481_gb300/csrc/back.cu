@@ -214,8 +214,9 @@ __device__ __forceinline__ void pixel_pair_tile(const T *__restrict__ b, int N, 
 // against FP64 is 6.6e-8 on smooth data and 7.4e-7 on white noise, 0.6 and 0.4
 // times that of one pixel per position from the tile's corner).
 // The raw bins are staged by 4-byte cp.async (rows have any alignment) one chunk
-// ahead.  Now bound by issue slots and the FMA pipe (about 4 issued instructions
-// per interpolation, 70 % of the slots): 512^2, 720 angles 73 -> 49 us (3.8 T
+// ahead.  Now bound by issue slots (about 4 issued instructions per
+// interpolation) and, at 512^2 with its 512 blocks, by latency at few warps (55 %
+// of the slots there): 512^2, 720 angles 73 -> 49 us (3.8 T
 // interpolations/s), 2048^2, 1800 angles 2,381 -> 1,399 us (5.4 T/s).
 constexpr int kBlkWarps = 4, kBlkThreads = 32 * kBlkWarps;
 constexpr int kBlkChunk = 16;         // angles per stage, two stages in flight
