@@ -4,6 +4,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include "proj_device.cuh"
@@ -192,7 +193,7 @@ __device__ __forceinline__ void pixel_pair_tile(const T *__restrict__ b, int N, 
     cluster.sync();   // peers' shared memory must outlive the reads above
 }
 
-// ---- 2 x 2 pixel blocks: the pixel-driven B for pitches of a pixel or more ----
+// ---- 2 x 2 pixel blocks: the pixel-driven B for pitches of a pixel or more (ctg_back_blocks_ok) ----
 // One interpolation per shared load is bound by the shared-memory data path
 // (8 bytes per interpolation, 16 interpolations per clock and SM).  Where one
 // pixel step moves at most one detector bin (|cos|, |sin| <= the pitch), a 2 x 2
@@ -221,9 +222,11 @@ __device__ __forceinline__ void pixel_pair_tile(const T *__restrict__ b, int N, 
 constexpr int kBlkWarps = 4, kBlkThreads = 32 * kBlkWarps;
 constexpr int kBlkChunk = 16;         // angles per stage, two stages in flight
 constexpr int kBlkFlush = 4;          // (1 in the smaller clusters: few angles, so few chains to average over)
-// Window of a 32 x th tile: a block's lowest corner lies within half the tile's
-// diagonal of the centre (21.92 bins for 32 rows, 35.11 for 64) plus a phase below
-// one, and reads the three bins after its own.
+// Window of a 32 x th tile: at a pitch of a pixel or more a block's lowest corner
+// lies within half the tile's diagonal of the centre (21.92 bins for 32 rows, 35.11
+// for 64) plus a phase below one, and reads the three bins after its own.  A finer
+// pitch whose angles all lie near a diagonal also has steps of at most one bin, but
+// up to 1.41 times the reach: ctg_back_blocks_ok asks for both.
 constexpr int blk_centre(int th) { return th <= 32 ? 24 : 37; }
 constexpr int blk_window(int th) { return th <= 32 ? 52 : 78; }
 
@@ -598,8 +601,21 @@ int blocks_for(int N, int split) {
 }  // namespace
 
 bool ctg_back_blocks_ok(const BackAngle *host_tab, int n_angles) {
-    for (int a = 0; a < n_angles; ++a)
-        if (!(fabsf(host_tab[a].cf) <= 1.0f && fabsf(host_tab[a].sf) <= 1.0f)) return false;
+    // a block spans at most 3 bins where a pixel step is at most one bin in
+    // either direction; its lowest corner is phase + oB j + oC i bins from the
+    // tile centre's bin, 0 <= phase < 1, j in [-15.5, 14.5] and i in [-(th - 1) / 2,
+    // (th - 3) / 2], and the window holds that bin and the next three.  Each bound
+    // has a 64th of a bin for the rounding of the positions.
+    constexpr double slack = 1.0 / 64;
+    for (int a = 0; a < n_angles; ++a) {
+        const double oB = std::fabs((double)host_tab[a].cf), oC = std::fabs((double)host_tab[a].sf);
+        if (!(oB <= 1.0 && oC <= 1.0)) return false;
+        for (const int th : {32, 64}) {
+            const double low = 0.5 * (kPT - 1) * oB + 0.5 * (th - 1) * oC;       // bins below the centre's phase
+            const double high = 1.0 + 0.5 * (kPT - 3) * oB + 0.5 * (th - 3) * oC; // and above its bin
+            if (low > blk_centre(th) - slack || high > blk_window(th) - 3 - blk_centre(th) - slack) return false;
+        }
+    }
     return true;
 }
 

@@ -178,7 +178,9 @@ void ctg_forward_plan(const FwdAngle *host_tab, int N, int n_angles, int n_det, 
 // angle, from the host copy of the angle table.
 int ctg_back_window(const BackAngle *host_tab, int n_angles);
 // Whether the pixel-driven B may take 2 x 2 pixel blocks: no angle moves more
-// than one detector bin per pixel step (every pitch of a pixel or more).
+// than one detector bin per pixel step, and every bin that a tile reads lies in
+// its staged window.  So at every pitch of a pixel or more, and at pitches just
+// below where all angles lie near the diagonals (at 45 degrees from 0.93 on).
 bool ctg_back_blocks_ok(const BackAngle *host_tab, int n_angles);
 // x = B b (+ add, if add != NULL); b has element type `dtype`; window from
 // ctg_back_window
