@@ -148,7 +148,7 @@ struct GeomEntry {
     FwdAngle *fwd = nullptr;
     BackAngle *back = nullptr;
     int back_window = 0;        // detector window of the tiled back projector
-    bool back_blocks = false;   // the pixel-driven B takes 2 x 2 pixel blocks
+    BackBlocks back_blocks = kBlocksNo;   // the pixel-driven B's 2 x 2 pixel blocks
     PadLayout pl{};             // staged-image layout of the forward projector
     float2 *pad = nullptr;      // context-owned staged image for ctg_project
     float2 *tw = nullptr;       // NCP: DFT twiddles of length n_det (on first use)
@@ -408,7 +408,7 @@ int tune_geometry(GeomEntry *ge) {
     const int back_cand[3] = {16, 32, 64};
     if (g->back_model == CTG_BACK_PIXEL)
         for (int c = 0; c < 3; ++c) {
-            if (c > 0 && ge->back_blocks) {         // its kernel has no pass size: one time for all three
+            if (c > 0 && ge->back_blocks != kBlocksNo) {         // its kernel has no pass size: one time for all three
                 ge->back_us[c] = ge->back_us[0];
                 continue;
             }
@@ -504,7 +504,7 @@ int get_geom(ctg_ctx *ctx, const ctg_geom *g, GeomEntry **out) {
     e.last_use = ++ctx->tick;
     e.serial = e.last_use;
     e.back_window = ctg_back_window(bk.data(), g->n_angles);
-    e.back_blocks = ctg_back_blocks_ok(bk.data(), g->n_angles);
+    e.back_blocks = ctg_back_blocks(bk.data(), g->n_angles);
     e.pl = ctg_pad_layout(g->N, g->det_spacing);
     cudaError_t err = cudaMalloc(&e.fwd, sizeof(FwdAngle) * fw.size());
     if (err == cudaSuccess) err = cudaMalloc(&e.back, sizeof(BackAngle) * bk.size());

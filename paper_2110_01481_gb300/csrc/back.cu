@@ -197,28 +197,32 @@ __device__ __forceinline__ void pixel_pair_tile(const T *__restrict__ b, int N, 
 // One interpolation per shared load is bound by the shared-memory data path
 // (8 bytes per interpolation, 16 interpolations per clock and SM).  Where one
 // pixel step moves at most one detector bin (|cos|, |sin| <= the pitch), a 2 x 2
-// block of pixels lies within [v, v + 1.42] bins of its lowest corner, so four
-// bins b0..b3 from floor(v) on serve all four pixels (and four reversed ones
-// their reflections): 4 bytes per interpolation, and one floor and one address
-// for eight.  With D = b1 - b0, K1 and K2 the second differences at b1 and b2, f
-// the corner's fraction and oB, oC the block's steps along its columns and rows,
-// the interpolant at f + o is
-//   b0 + D f + D o + K1 max(0, f + o - 1) + K2 max(0, f + o - 2),
-// so over the angles the four pixels share the sums S = sum (b0 + D f), G =
-// sum D oB, H = sum D oC: corner S, next column B = S + G + sum K1 r1(oB), next
-// row C = S + H + sum K1 r1(oC), far corner E = S + G + H + sum (K1 r1(oB + oC) +
-// K2 r2(oB + oC)) (K2 enters only there, as oB, oC <= 1).
+// block of pixels lies within three bins of its lowest corner, so four bins
+// b0..b3 from floor(v) on serve all four pixels (and four reversed ones their
+// reflections): 4 bytes per interpolation, and one floor and one address for
+// eight.  A pixel at t bins from bin j takes b[j-1], b[j], b[j+1] with the weights
+// max(0, -t), 1 - |t| and max(0, t) for |t| <= 1, so with the corner's fraction f
+// and oB, oC the block's steps along its columns and rows: the corner takes b0
+// and b1 with 1 - f and f, the next column and the next row lie at f + oB - 1 and
+// f + oC - 1 from b1, and the far corner at f + oB + oC - 2 from b2 where oB + oC
+// >= 1 (kUnit; at every angle for a pitch of a pixel, ctg_back_blocks_unit), else
+// it takes all four bins.  A bin that a pixel does not interpolate has the weight
+// zero exactly, so a large value leaves nothing in its neighbours.  (First and
+// second differences from b0, shared by the four pixels, are 2 % faster, but carry
+// the rounding of every bin of the four: a bin of 1e6 in unit noise left 0.6 in
+// pixels beside its reach at 64^2, 90 angles and 1.1 at 512^2, now 3e-5 and 1.4e-4,
+// what the noise alone leaves.)
 // An angle with sin < 0 is taken as its opposite (the reversed projection), so
 // the lowest corner is the left column for cos >= 0 and the right one for cos
 // < 0; the sums go to the pixels when that changes, and every kBlkFlush chunks
 // (which also keeps the chains of additions short: at 512^2, 720 angles the error
-// against FP64 is 6.6e-8 on smooth data and 7.4e-7 on white noise, 0.6 and 0.4
-// times that of one pixel per position from the tile's corner).
+// against FP64 is 6.6e-8 on smooth data and 1.1e-6 on white noise, 0.6 times that
+// of one pixel per position from the tile's corner).
 // The raw bins are staged by 4-byte cp.async (rows have any alignment) one chunk
-// ahead.  Now bound by issue slots (about 4 issued instructions per
-// interpolation) and, at 512^2 with its 512 blocks, by latency at few warps (55 %
-// of the slots there): 512^2, 720 angles 73 -> 49 us (3.8 T
-// interpolations/s), 2048^2, 1800 angles 2,381 -> 1,399 us (5.4 T/s).
+// ahead.  Now bound by issue slots (about 4.5 issued instructions per
+// interpolation) and, at 512^2 with its 512 blocks, by latency at few warps:
+// 512^2, 720 angles 73.5 -> 51.3 us (3.7 T interpolations/s), 2048^2, 1800 angles
+// 2,383 -> 1,437 us (5.3 T/s); 50.4 and 1,414 us with the differences.
 constexpr int kBlkWarps = 4, kBlkThreads = 32 * kBlkWarps;
 constexpr int kBlkChunk = 16;         // angles per stage, two stages in flight
 constexpr int kBlkFlush = 4;          // (1 in the smaller clusters: few angles, so few chains to average over)
@@ -230,19 +234,6 @@ constexpr int kBlkFlush = 4;          // (1 in the smaller clusters: few angles,
 constexpr int blk_centre(int th) { return th <= 32 ? 24 : 37; }
 constexpr int blk_window(int th) { return th <= 32 ? 52 : 78; }
 
-__device__ __forceinline__ float sat_add(float a, float b) { return __saturatef(a + b); }
-
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
-    float2 r;
-    asm("{\n\t.reg .b64 a, b, r;\n\t"
-        "mov.b64 a, {%2, %3};\n\t"
-        "mov.b64 b, {%4, %5};\n\t"
-        "sub.rn.f32x2 r, a, b;\n\t"
-        "mov.b64 {%0, %1}, r;\n\t}"
-        : "=f"(r.x), "=f"(r.y)
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-    return r;
-}
 // acc += a * (s, s)
 __device__ __forceinline__ void fma2s(float2 &acc, float2 a, float s) {
     asm("{\n\t.reg .b64 c, a, s;\n\t"
@@ -254,15 +245,17 @@ __device__ __forceinline__ void fma2s(float2 &acc, float2 a, float s) {
         : "+f"(acc.x), "+f"(acc.y)
         : "f"(a.x), "f"(a.y), "f"(s));
 }
-__device__ __forceinline__ void fma_each(float2 &acc, float2 a, float s) {
-    acc.x = fmaf(a.x, s, acc.x);
-    acc.y = fmaf(a.y, s, acc.y);
+// acc += the interpolation at t from the middle one of three bins, |t| <= 1
+__device__ __forceinline__ void three_bins(float2 &acc, float2 lo, float2 mid, float2 hi, float t) {
+    fma2s(acc, lo, fmaxf(-t, 0.0f));
+    fma2s(acc, mid, 1.0f - fabsf(t));
+    fma2s(acc, hi, fmaxf(t, 0.0f));
 }
 
 // The CTA's pixel sums for angles [a_begin, a_end) one interpolation at a time,
 // from global memory: taken when the block sums hold a value that is not
-// finite, because a second difference would carry an infinite or NaN bin (or
-// the overflow of a difference) to neighbours that do not interpolate it.
+// finite, because a weight of zero would carry an infinite or NaN bin to
+// neighbours that do not interpolate it.
 template <typename T>
 __device__ __noinline__ void pixel_back_plain(const T *__restrict__ b, int n_det, const BackAngle *__restrict__ tab,
                                               int a_begin, int a_end, int j0, int i0, int rows, float *s_px) {
@@ -284,7 +277,7 @@ __device__ __noinline__ void pixel_back_plain(const T *__restrict__ b, int n_det
 // Body of one CTA of the cluster for the 32 x (16 kNB) tile (bx, by) of the
 // upper half; each of the 128 threads owns kNB blocks 16 rows apart.  Every CTA
 // of a cluster must call it.
-template <typename T, int kNB, int kSplit>
+template <typename T, int kNB, int kSplit, bool kUnit>
 __device__ __forceinline__ void pixel_back_blocks(const T *__restrict__ b, int N, int n_angles, int n_det,
                                                   const BackAngle *__restrict__ tab,
                                                   const float *__restrict__ add, float *__restrict__ x, int bx,
@@ -362,10 +355,10 @@ __device__ __forceinline__ void pixel_back_blocks(const T *__restrict__ b, int N
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
 
-    float2 S[kNB], G[kNB], H[kNB], B[kNB], C[kNB], E[kNB];
+    float2 A[kNB], B[kNB], C[kNB], E[kNB];             // lowest corner, next column, next row, far corner
     auto clear = [&] {
 #pragma unroll
-        for (int q = 0; q < kNB; ++q) S[q] = G[q] = H[q] = B[q] = C[q] = E[q] = make_float2(0.f, 0.f);
+        for (int q = 0; q < kNB; ++q) A[q] = B[q] = C[q] = E[q] = make_float2(0.f, 0.f);
     };
     auto flush = [&](bool right) {
 #pragma unroll
@@ -374,9 +367,7 @@ __device__ __forceinline__ void pixel_back_blocks(const T *__restrict__ b, int N
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 auto at = [&](const float2 &v) { return h ? v.y : v.x; };
-                const float a = at(S[q]), bb = (at(S[q]) + at(G[q])) + at(B[q]);
-                const float cc = (at(S[q]) + at(H[q])) + at(C[q]);
-                const float ee = (at(S[q]) + (at(G[q]) + at(H[q]))) + at(E[q]);
+                const float a = at(A[q]), bb = at(B[q]), cc = at(C[q]), ee = at(E[q]);
                 float2 *p0 = reinterpret_cast<float2 *>(s_px + (h * kTH + row) * kPT + col);
                 float2 *p1 = reinterpret_cast<float2 *>(s_px + (h * kTH + row + 1) * kPT + col);
                 float2 t0 = *p0, t1 = *p1;
@@ -423,7 +414,7 @@ __device__ __forceinline__ void pixel_back_blocks(const T *__restrict__ b, int N
                 right = r;
                 sdj = r ? -(fdj + 1.0f) : fdj;
             }
-#pragma unroll 2
+#pragma unroll 4
             for (; k < end; ++k, sb += 8u * kWin) {
                 const float4 p = par[k][0], o = par[k][1];
                 const float u0 = fmaf(p.z, fdi, fmaf(p.y, sdj, p.x));
@@ -438,16 +429,20 @@ __device__ __forceinline__ void pixel_back_blocks(const T *__restrict__ b, int N
                     const float2 *e = static_cast<const float2 *>(__cvta_shared_to_generic(at));
                     const float2 b0 = e[0], b1 = e[1], b2 = e[2], b3 = e[3];
                     const float f = ff[q];
-                    const float2 D0 = sub2(b1, b0), D1 = sub2(b2, b1), D2 = sub2(b3, b2);
-                    const float2 K1 = sub2(D1, D0), K2 = sub2(D2, D1);
-                    add2(S[q].x, S[q].y, b0.x, b0.y);
-                    fma_each(S[q], D0, f);
-                    fma2s(G[q], D0, p.y);
-                    fma2s(H[q], D0, p.z);
-                    fma_each(B[q], K1, sat_add(f, p.w));
-                    fma_each(C[q], K1, sat_add(f, o.x));
-                    fma_each(E[q], K1, fmaxf(f + o.y, 0.0f));
-                    fma_each(E[q], K2, sat_add(f, o.z));
+                    fma2s(A[q], b0, 1.0f - f);
+                    fma2s(A[q], b1, f);
+                    const float tB = f + p.w, tC = f + o.x, tE = f + o.z;
+                    three_bins(B[q], b0, b1, b2, tB);
+                    three_bins(C[q], b0, b1, b2, tC);
+                    if constexpr (kUnit) {
+                        three_bins(E[q], b1, b2, b3, tE);
+                    } else {
+                        const float t = f + o.y;            // from b1, tE from b2
+                        fma2s(E[q], b0, fmaxf(-t, 0.0f));
+                        fma2s(E[q], b1, __saturatef(1.0f - fabsf(t)));
+                        fma2s(E[q], b2, __saturatef(1.0f - fabsf(tE)));
+                        fma2s(E[q], b3, fmaxf(tE, 0.0f));
+                    }
                 }
             }
         }
@@ -491,13 +486,13 @@ constexpr size_t blk_smem(int nb) {
 }
 constexpr int blk_tiles_y(int N, int nb) { return ((N + 1) / 2 + 16 * nb - 1) / (16 * nb); }
 
-template <typename T, int kNB, int kSplit>
+template <typename T, int kNB, int kSplit, bool kUnit>
 __global__ void __cluster_dims__(1, 1, kSplit) __launch_bounds__(kBlkThreads, kNB == 4 ? 4 : 7)
 pixel_back_blocks_kernel(const T *__restrict__ b, ColRef bc, int N, int n_angles, int n_det,
                          const BackAngle *__restrict__ tab, const float *__restrict__ add, float *__restrict__ x,
                          const SolveIo *__restrict__ io) {
     if (io) add = io->x0, x = io->x;
-    pixel_back_blocks<T, kNB, kSplit>(b + col_offset(bc), N, n_angles, n_det, tab, add, x, blockIdx.x, blockIdx.y);
+    pixel_back_blocks<T, kNB, kSplit, kUnit>(b + col_offset(bc), N, n_angles, n_det, tab, add, x, blockIdx.x, blockIdx.y);
 }
 
 // bc: the input is column bc of a basis (b + col_offset(bc)), or b itself.
@@ -619,6 +614,17 @@ bool ctg_back_blocks_ok(const BackAngle *host_tab, int n_angles) {
     return true;
 }
 
+bool ctg_back_blocks_unit(const BackAngle *host_tab, int n_angles) {
+    // the far corner's distance from b2, f + (oB - 1) + (oC - 1), must not round
+    // to below -1: a margin, or an angle along an axis, whose steps are exact
+    for (int a = 0; a < n_angles; ++a) {
+        const double oB = std::fabs((double)host_tab[a].cf), oC = std::fabs((double)host_tab[a].sf);
+        const bool axis = (oB == 1.0 && oC == 0.0) || (oB == 0.0 && oC == 1.0);
+        if (!axis && !(oB + oC >= 1.0 + 1e-6)) return false;
+    }
+    return true;
+}
+
 namespace {
 
 // The arguments of one back projection.
@@ -645,24 +651,28 @@ void launch_pair(const BackArgs<T> &a) {
 }
 
 template <int kNB, int kSplit, typename T>
-void launch_blocks(const BackArgs<T> &a) {
+void launch_blocks(const BackArgs<T> &a, bool unit) {
     const dim3 grid(back_tiles_x(a.N), blk_tiles_y(a.N, kNB), kSplit);
-    pixel_back_blocks_kernel<T, kNB, kSplit><<<grid, kBlkThreads, blk_smem(kNB), a.st>>>(
-        a.b, a.bc, a.N, a.n_angles, a.n_det, a.tab, a.add, a.x, a.io);
+    auto run = [&](auto kernel) {
+        kernel<<<grid, kBlkThreads, blk_smem(kNB), a.st>>>(a.b, a.bc, a.N, a.n_angles, a.n_det, a.tab, a.add, a.x, a.io);
+    };
+    if (unit) run(pixel_back_blocks_kernel<T, kNB, kSplit, true>);
+    else run(pixel_back_blocks_kernel<T, kNB, kSplit, false>);
 }
 
-// blocks: the 2 x 2 block kernel (ctg_back_blocks_ok).  back_chunk: angles
+// blocks: the 2 x 2 block kernel and its form.  back_chunk: angles
 // staged per pass of the one-pixel tiled kernel, 16 or (any other value, where
 // it fits) 32.  Each pixel sums its angles in the same order whatever the
 // chunk, so the result does not depend on it.
 template <typename T>
-cudaError_t launch_back_t(const BackArgs<T> &a, bool blocks, int back_chunk) {
-    if (blocks) {
+cudaError_t launch_back_t(const BackArgs<T> &a, BackBlocks blocks, int back_chunk) {
+    if (blocks != kBlocksNo) {
+        const bool unit = blocks == kBlocksUnit;
         const int split = split_for(a.n_angles, back_tiles_x(a.N) * blk_tiles_y(a.N, 2));
         const bool four = blocks_for(a.N, split) == 4;
-        if (split == 8) four ? launch_blocks<4, 8>(a) : launch_blocks<2, 8>(a);
-        else if (split == 4) four ? launch_blocks<4, 4>(a) : launch_blocks<2, 4>(a);
-        else four ? launch_blocks<4, 2>(a) : launch_blocks<2, 2>(a);
+        if (split == 8) four ? launch_blocks<4, 8>(a, unit) : launch_blocks<2, 8>(a, unit);
+        else if (split == 4) four ? launch_blocks<4, 4>(a, unit) : launch_blocks<2, 4>(a, unit);
+        else four ? launch_blocks<4, 2>(a, unit) : launch_blocks<2, 2>(a, unit);
     } else if (a.window > 0 && a.window <= kBackWindowMaxTiled) {
         // four rows per thread (a finer pitch's windows leave room for few
         // CTAs); two CTAs per cluster once that fills the device (pitch 0.75:
@@ -720,7 +730,7 @@ cudaError_t ctg_launch_back_matched_tiled(const void *b, int dtype, int N, int n
 }
 
 cudaError_t ctg_launch_back(const void *b, int dtype, int N, int n_angles, int n_det,
-                            const BackAngle *tab, int window, bool blocks, const float *add, float *x,
+                            const BackAngle *tab, int window, BackBlocks blocks, const float *add, float *x,
                             cudaStream_t st, int back_chunk, ColRef bc, const SolveIo *io) {
     auto run = [&](auto *p) {
         using T = typename std::remove_const<typename std::remove_pointer<decltype(p)>::type>::type;

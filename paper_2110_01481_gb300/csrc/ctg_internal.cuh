@@ -180,16 +180,25 @@ int ctg_back_window(const BackAngle *host_tab, int n_angles);
 // Whether the pixel-driven B may take 2 x 2 pixel blocks: no angle moves more
 // than one detector bin per pixel step, and every bin that a tile reads lies in
 // its staged window.  So at every pitch of a pixel or more, and at pitches just
-// below where all angles lie near the diagonals (at 45 degrees from 0.93 on).
+// below where all angles lie near the diagonals (at 45 degrees from 0.92 on).
 bool ctg_back_blocks_ok(const BackAngle *host_tab, int n_angles);
+// Whether a block's far corner lies at least one bin beyond its lowest one at
+// every angle (so at every pitch up to a pixel that takes blocks).
+bool ctg_back_blocks_unit(const BackAngle *host_tab, int n_angles);
+// The form of the block kernel for a table: none, four bins for the far corner, or three.
+enum BackBlocks { kBlocksNo = 0, kBlocksGeneral, kBlocksUnit };
+static inline BackBlocks ctg_back_blocks(const BackAngle *host_tab, int n_angles) {
+    if (!ctg_back_blocks_ok(host_tab, n_angles)) return kBlocksNo;
+    return ctg_back_blocks_unit(host_tab, n_angles) ? kBlocksUnit : kBlocksGeneral;
+}
 // x = B b (+ add, if add != NULL); b has element type `dtype`; window from
 // ctg_back_window
-// blocks: ctg_back_blocks_ok's answer for the table.
+// blocks: ctg_back_blocks' answer for the table.
 // back_chunk: angles staged per pass, 16, 32 or 64 (tuned like the forward shape;
 // the result does not depend on it, and the block kernel does not use it).
 // bc: the input is column bc of a basis at b (bc.k set), or b itself.
 cudaError_t ctg_launch_back(const void *b, int dtype, int N, int n_angles, int n_det,
-                            const BackAngle *tab, int window, bool blocks, const float *add, float *x,
+                            const BackAngle *tab, int window, BackBlocks blocks, const float *add, float *x,
                             cudaStream_t st, int back_chunk = 32, ColRef bc = col_none(),
                             const SolveIo *io = nullptr);     // io: add = io->x0, x = io->x
 

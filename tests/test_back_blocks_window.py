@@ -90,3 +90,28 @@ def test_every_index_lies_in_the_staged_window(blocks_ok, N, ds):
                 assert least >= 0 and most < window, (start, range_, n_angles, nd, rows, least, most)
     if ds >= 1.0:
         assert admitted == 2 * len(SCANS)                   # every scan at a pitch of a pixel or more
+
+
+def test_far_corner_rule(blocks_ok):
+    """Where the far corner takes three bins (one bin or more beyond the lowest
+    corner), its distance f + (oB - 1) + (oC - 1) from the middle one of them,
+    formed in FP32, lies in [-1, 1] for every fraction f in [0, 1)."""
+    from paper_2110_01481_gb300 import _native
+    unit = ctypes.CDLL(_native.LIB_PATH)["_Z20ctg_back_blocks_unitPK9BackAnglei"]     # ctg_back_blocks_unit(table, angles)
+    unit.restype, unit.argtypes = ctypes.c_bool, [ctypes.POINTER(BackAngle), ctypes.c_int]
+    f32 = np.float32
+    seen = set()
+    for ds, (start, range_, n_angles) in itertools.product(PITCHES + [1.2, 1.4, 1.0000001, 2.0], SCANS + [(0, 360, 100000)]):
+        tab = _table(64, n_angles, 91, start, range_, ds)
+        if not blocks_ok(tab, n_angles):
+            continue
+        is_unit = unit(tab, n_angles)
+        seen.add((ds > 1.0, is_unit))
+        if is_unit:
+            for t in tab:
+                oB, oC = abs(f32(t.cf)), abs(f32(t.sf))
+                o = f32(f32(oB - f32(1)) + f32(oC - f32(1)))
+                assert f32(f32(0) + o) >= -1.0 and f32(f32(1 - 2.0 ** -24) + o) <= 1.0
+        elif ds == 1.0:
+            raise AssertionError((start, range_, n_angles))
+    assert seen == {(False, True), (True, True), (True, False)}
