@@ -220,7 +220,7 @@ int ctg_workspace_layout(const ctg_geom *g, int variant, const ctg_opts *o,
  * workspace: device memory of >= workspace_bytes bytes, 256-byte aligned, or
  * NULL, in which case the library takes it from a memory pool of the
  * context per call, in stream order (the pool keeps up to 512 MiB between
- * calls, until ctg_destroy).  The
+ * calls, until ctg_release_memory or ctg_destroy).  The
  * caller owns b, x0, x and the workspace; none may alias another.  Runs on
  * `stream`, synchronises it before returning and fills *info (info may not
  * be NULL).  A breakdown (h_{k+1,k} <= 1e-6 ||A B w_k||) is reported in
@@ -397,6 +397,13 @@ int ctg_cgs2_noalloc(const float *W_dev, int64_t ld_w, int64_t L, int32_t k,
  * arrived, which tests use to exercise this path.  Takes effect at the next
  * solve. */
 int ctg_set_wait_limit(ctg_ctx *ctx, int64_t polls);
+
+/* Gives back to the device the memory that the context's pool keeps between
+ * solves (the paper has no counterpart).  Nothing of it holds a result; the
+ * next solve with a library workspace maps its memory anew.  Needed before
+ * another process or API is to have that memory: an allocation of this
+ * process that the device cannot serve otherwise gets it from the driver. */
+int ctg_release_memory(ctg_ctx *ctx);
 
 /* Phase tracing (the paper has no counterpart; it reports no timings).
  * When enabled, the solvers bracket each phase with CUDA events on the

@@ -84,6 +84,11 @@ class Context:
         then raises CtgError with CTG_ERR_TIMEOUT); 0 restores the default."""
         nat.check(nat.lib().ctg_set_wait_limit(self.handle, int(polls)), "ctg_set_wait_limit")
 
+    def release_memory(self) -> None:
+        """Give back the device memory (up to 512 MiB) that is kept between
+        solves without a caller's workspace."""
+        nat.check(nat.lib().ctg_release_memory(self.handle), "ctg_release_memory")
+
     def set_tiles(self, fwd_angles: int = 0, back_chunk: int = 0, fwd_warp_angles: int = 1) -> None:
         """Force the projectors' tile shapes (0, 0: autotuned per geometry).
         The forward shape is fwd_angles angles per block with fwd_warp_angles

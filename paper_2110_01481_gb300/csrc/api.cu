@@ -768,7 +768,9 @@ struct SolveCtx {
 // default pool gives its memory back to the device at every synchronisation,
 // which made each solve map its workspace anew: 110 us at 64^2 to 370 us at
 // 512^2 of a solve's time.  The pool here keeps up to kPoolKeep bytes until
-// ctg_destroy (a solve that needs more has seconds of device work), and a
+// ctg_release_memory or ctg_destroy (a solve that needs more has seconds of
+// device work; an allocation of this process that the device cannot serve
+// otherwise gets them from the driver), and a
 // workspace mostly gets its last address again, so that the loop captured
 // with it is found again too.  With the current device not the pool's, or no
 // pool to be had, the default pool serves.
@@ -1441,6 +1443,12 @@ void ctg_destroy(ctg_ctx *ctx) {
     if (ctx->ev_init) cudaEventDestroy(ctx->ev_init);
     if (ctx->pinned) cudaFreeHost(ctx->pinned);
     delete ctx;
+}
+
+int ctg_release_memory(ctg_ctx *ctx) {
+    if (!ctx) return CTG_ERR_INVALID_ARG;
+    if (ctx->pool) CTG_CK(cudaMemPoolTrimTo(ctx->pool, 0));
+    return CTG_OK;
 }
 
 int ctg_set_wait_limit(ctg_ctx *ctx, int64_t polls) {
