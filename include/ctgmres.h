@@ -162,10 +162,11 @@ int ctg_backproject(ctg_ctx *ctx, const ctg_geom *g, const float *b_dev,
  * a geometry, the forward projector with 8 and 4 angles per block (one angle
  * per warp, 32 adjacent rays) and with 8 and 16 angles per block (4 angles
  * per warp, 8 adjacent rays of each), and the pixel-driven back projector
- * with 16, 32 and 64 angles staged per pass (CUDA events, 3 launches each on
- * zero inputs, with temporary buffers of about 5n + m floats), and keeps the
- * fastest (at a pitch of a pixel or more the back projector has one form,
- * timed once).  The shapes with 4 angles per warp are candidates only where the
+ * with 16 and 32 angles staged per pass (CUDA events, 3 launches each on zero
+ * inputs, with temporary buffers of about 5n + m floats), and keeps the
+ * fastest.  (64 is accepted: batches stage that many, a single launch then
+ * 32.  At a pitch of a pixel or more the back projector has one form; what
+ * launches the same kernel is timed once.)  The shapes with 4 angles per warp are candidates only where the
  * host has checked that every warp's walk stays inside the staged image
  * (adjacent angles of a fine angular sampling; not widely spaced ones).  The
  * candidates sum every ray and every pixel in the same order, so results do
@@ -183,7 +184,7 @@ typedef struct {
     int32_t back_chunk;       /* 16, 32 or 64                               */
     int32_t tuned;            /* 1 if chosen by timing                      */
     float fwd_us[2];          /* measured: 8, 4 angles per block, 1 per warp */
-    float back_us[3];         /* measured: 16, 32, 64 angles per pass       */
+    float back_us[3];         /* measured: 16, 32, 64 (as 32) angles per pass */
     int32_t fwd_warp_angles;  /* angles per warp of the forward shape: 1, 4 */
     float fwd_split_us[2];    /* measured: 8, 16 angles per block, 4 per warp */
 } ctg_tuning;

@@ -408,8 +408,11 @@ int tune_geometry(GeomEntry *ge) {
     const int back_cand[3] = {16, 32, 64};
     if (g->back_model == CTG_BACK_PIXEL)
         for (int c = 0; c < 3; ++c) {
-            if (c > 0 && ge->back_blocks != kBlocksNo) {         // its kernel has no pass size: one time for all three
-                ge->back_us[c] = ge->back_us[0];
+            auto used = [&](int d) { return ctg_back_chunk_used(ge->back_blocks, ge->back_window, back_cand[d]); };
+            int same = 0;                           // a pass size that launches the same kernel is timed once
+            while (used(same) != used(c)) ++same;
+            if (same < c) {
+                ge->back_us[c] = ge->back_us[same];
                 continue;
             }
             timed([&] {

@@ -614,6 +614,11 @@ bool ctg_back_blocks_ok(const BackAngle *host_tab, int n_angles) {
     return true;
 }
 
+int ctg_back_chunk_used(BackBlocks blocks, int window, int chunk) {
+    const bool pairs = blocks == kBlocksNo && window > 0 && window <= kBackWindowMaxTiled;
+    return pairs ? back_chunk_for(chunk, window) : 0;
+}
+
 bool ctg_back_blocks_unit(const BackAngle *host_tab, int n_angles) {
     // the far corner's distance from b2, f + (oB - 1) + (oC - 1), must not round
     // to below -1: a margin, or an angle along an axis, whose steps are exact

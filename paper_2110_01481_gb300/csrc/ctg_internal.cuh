@@ -194,9 +194,11 @@ static inline BackBlocks ctg_back_blocks(const BackAngle *host_tab, int n_angles
 // x = B b (+ add, if add != NULL); b has element type `dtype`; window from
 // ctg_back_window
 // blocks: ctg_back_blocks' answer for the table.
-// back_chunk: angles staged per pass, 16, 32 or 64 (tuned like the forward shape;
-// the result does not depend on it, and the block kernel does not use it).
+// back_chunk: angles staged per pass, 16 or (any other value) 32, fewer where the
+// windows are wide (tuned like the forward shape; the result does not depend on
+// it, and only the pixel pairs use it: ctg_back_chunk_used, 0 for the other kernels).
 // bc: the input is column bc of a basis at b (bc.k set), or b itself.
+int ctg_back_chunk_used(BackBlocks blocks, int window, int chunk);
 cudaError_t ctg_launch_back(const void *b, int dtype, int N, int n_angles, int n_det,
                             const BackAngle *tab, int window, BackBlocks blocks, const float *add, float *x,
                             cudaStream_t st, int back_chunk = 32, ColRef bc = col_none(),
