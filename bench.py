@@ -174,9 +174,10 @@ def joseph_interpolations(N, n_angles, n_det, start=0, rng=180, ds=1.0):
 
 
 def l1_peak(torch, dev, sm_max_mhz):
-    """SM-side bound of the projectors: every interpolation moves one 8-byte
-    (value, difference) pair through the SM's L1/shared data path, 128 B/clk
-    per SM, on the device's SM count (queried: 152 on a GB300) at its maximum
+    """SM-side bound of the projectors: every interpolation of A moves one
+    8-byte (value, difference) pair through the SM's L1/shared data path, every
+    one of B 4 bytes (2 x 2 pixel blocks and their reflections), 128 B/clk per
+    SM, on the device's SM count (queried: 152 on a GB300) at its maximum
     SM clock (sampled by nvidia-smi; 2070 MHz on a GB300).  GB/s."""
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     mhz = sm_max_mhz if sm_max_mhz else 2070.0
@@ -837,7 +838,7 @@ def run_gpu(args):
     phases = {p: tm[p] for p in _native.PHASES}
     arnoldi_roof = {
         "bound": "hbm", "unit": "GB/s",
-        "kernel": "CGS2 Arnoldi step (one cooperative launch up to k = 128 when its grid fits, else 3 passes)",
+        "kernel": "CGS2 Arnoldi step (one cooperative launch up to k = 128 when its grid fits and, for ctg_cgs2, the basis is below 300 MB, else 3 passes)",
         "achieved": arn_bytes / (phases["arnoldi"]["ms"] / 1e3) / 1e9 if phases["arnoldi"]["ms"] else None,
         "peak": hbm, "peak_kind": peak_kind + " copy bandwidth",
     }
@@ -855,16 +856,18 @@ def run_gpu(args):
         if dom == "forward":
             interp = joseph_interpolations(N, N_ANG, N_DET)
             kname = "joseph_forward_kernel"
+            per_interp, what = 8.0, "one value/difference pair"
         else:
             interp = n * N_ANG
             kname = "pixel_back_blocks_kernel"
+            per_interp, what = 4.0, "four bins and their reflections, 32 B, serve eight"
         per_launch_s = phases[dom]["ms"] / 1e3 / phases[dom]["calls"]
-        ach = 8.0 * interp / per_launch_s / 1e9
+        ach = per_interp * interp / per_launch_s / 1e9
         l1, sms, mhz = l1_peak(torch, dev, clocks.get("sm_max_mhz"))
         roof = {"bound": "alu", "unit": "GB/s", "kernel": kname,
                 "achieved": ach, "peak": l1,
                 "peak_kind": f"derived: L1/shared data path, {sms} SM (queried) x 128 B/clk x "
-                             f"{mhz / 1e3:.3f} GHz (max SM clock); 8 B (one value/difference pair) "
+                             f"{mhz / 1e3:.3f} GHz (max SM clock); {per_interp:.0f} B ({what}) "
                              "per interpolation",
                 "frac": ach / l1, "traffic": recorded_traffic(kname),
                 "interpolations_per_launch": interp,

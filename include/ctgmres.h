@@ -389,8 +389,8 @@ int ctg_cgs2_noalloc(const float *W_dev, int64_t ld_w, int64_t L, int32_t k,
 /* Bounded device-side waits (the paper has no counterpart).  The one-launch
  * CGS2 step of the solvers separates its passes with grid-wide barriers,
  * which rely on every block of the launch being resident.  Each wait polls
- * at most `polls` times (about 100 ns apart; 0 restores the default of
- * 2^22, about half a second) and then gives up: the solve stops and
+ * at most `polls` times (about 0.34 us apart; 0 restores the default of
+ * 2^22, about a second and a half) and then gives up: the solve stops and
  * ctg_ab_gmres / ctg_ba_gmres return CTG_ERR_TIMEOUT (the context stays
  * usable; x then holds no meaningful iterate).  The batched one-launch step
  * of ctg_batch_solve, for batches created on this context, takes the same

@@ -1,8 +1,6 @@
 // C-ABI of libctgmres (declared in include/ctgmres.h): geometry tables,
-// workspace layout and the host loops of AB-GMRES and BA-GMRES (paper
-// Sec. 2, algorithm box), with the Hessenberg least-squares problem solved
-// by FP64 Givens rotations on the host and the discrepancy-principle stop
-// of Sec. 6.4.
+// workspace layout, the AB-GMRES and BA-GMRES solves (paper Sec. 2, algorithm
+// box) as loops that run on the device, and the host loops of LSQR and LSMR.
 #include <cmath>
 #include <cstdio>
 #include <algorithm>

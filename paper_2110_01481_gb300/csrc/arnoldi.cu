@@ -4,7 +4,7 @@
 // (CGS2), which equals the paper's MGS loop in exact arithmetic but needs
 // three sweeps over W instead of k dependent ones:
 //   pass 1  h1 = W^T q,                ||q||^2      (one read of W)
-//   pass 2  q -= W h1,  h2 = W^T q,    ||q1||^2     (two reads of W, or one: cgs_sweep_kernel)
+//   pass 2  q -= W h1,  h2 = W^T q,    ||q1||^2     (two reads of W; one by cgs_sweep_kernel in a caller's own loop)
 //   pass 3  q -= W h2,  w_{k+1} = q / ||q||         (one read of W)
 // with ||q||^2 = ||q1||^2 - ||h2||^2 after pass 3 (exact for orthonormal W;
 // h2 is at the rounding level of ||q1|| after the first pass, so nothing
@@ -351,7 +351,7 @@ __device__ __forceinline__ void write_rows(const float *s_w, int nred, int row0,
 // with a bounded wait: thread 0 of each block adds one arrival to *count
 // and waits until `target` arrivals are in (target = barrier index x grid
 // size, so one counter serves successive barriers).  After spin_limit polls
-// (some 400 ns apart) it gives up: it sets *err and returns false, as does
+// (0.34 us apart) it gives up: it sets *err and returns false, as does
 // every block that finds *err set while it waits, so no block waits for
 // ever.  Returns true when the barrier completed.
 __device__ __forceinline__ bool grid_barrier(unsigned *count, unsigned target, long long spin_limit,
@@ -1273,6 +1273,9 @@ cudaError_t fused_dispatch(const T *W, int64_t ldw, int64_t L, int k, float *q, 
 // time against cgs_pass_kernel's two reads (us): L = 2.4M, k = 12 (115 MB)
 // 26 / 30; 522,000 x 60 (125 MB) 27 / 31; 522,000 x 40 (84 MB) 23 / 21;
 // 4.19M x 8 36 / 40 and x 4 34 / 20; 131,072 x 150 28 / 34; 4,099 x 200 16 / 42.
+// Steps of ctg_cgs2 and ctg_cgs2_noalloc take it; those of the solvers' captured
+// loops and of batches, where k is read on the device while this kernel's shape
+// and ring are chosen by k at the launch, keep the two reads.
 constexpr int kSweepMinK = 8, kSweepMaxK = 216;
 constexpr int64_t kSweepMinBytes = 100000000;
 // From 300 MB on, the passes with it are faster than the one-launch step with

@@ -255,8 +255,8 @@ static inline size_t ctg_basis_bytes(int dtype) {
     return dtype == CTG_BASIS_FP32 ? 4 : (dtype == CTG_BASIS_BF16 || dtype == CTG_BASIS_FP16) ? 2 : 0;
 }
 
-// Polls of a bounded device-side wait (about 100 ns apart) before it gives
-// up: about half a second.
+// Polls of a bounded device-side wait (0.34 us apart, measured with one block
+// polling) before it gives up: about a second and a half.
 constexpr long long kCtgDefaultSpinLimit = 1LL << 22;
 
 // One CGS2 Arnoldi step: orthogonalise the FP32 vector q (length L) against

@@ -21,9 +21,9 @@ __device__ __forceinline__ float fx_frac(long long U) {
 }
 
 // floor(u) by the round-down magic-number add, for two positions at once in
-// packed FP32 pairs: t = u + M rounded down (M = 1.5 * 2^23, so the low
-// mantissa bits of t hold floor(u) for 0 <= u < 2^22) and f = u - (t - M),
-// exactly the scalar sequence per position, with half the instructions.
+// packed FP32 pairs: t = u + M rounded down (M = 1.5 * 2^23, so the bits of t
+// are those of M plus floor(u), negative ones too, for |u| < 2^22) and f = u -
+// (t - M), exactly the scalar sequence per position, with half the instructions.
 __device__ __forceinline__ void floor_frac2(float u0, float u1, float &t0, float &t1, float &f0,
                                             float &f1) {
     asm("{\n\t.reg .b64 u, m, t, f;\n\t"

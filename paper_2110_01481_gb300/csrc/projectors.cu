@@ -286,11 +286,13 @@ joseph_forward_kernel(const void *__restrict__ pad, int N, int stride, int borde
 
 // ---------------------------------------------------------------------------
 // Back projection of batched and served solves.  (Single launches have faster
-// kernels, back.cu.  Their positions and sums round differently, about 1e-7
-// of B b; a solve of a batch may run to steps where the iterate is an
-// ill-conditioned function of the rounding and moves by 1e-3, so batches keep
-// this kernel's sums: measured with the 2 x 2 block kernel in its place,
-// iterates at k >= 20 moved by up to 5e-3 for 10 % of the time.)
+// kernels, back.cu, which round differently, about 1e-7 of B b, and are nearer to
+// FP64.  This one stays so that batched results stay bit for bit what they were:
+// with the 2 x 2 block kernel in its place a batch was 10 % faster, iterates of
+// 10 early steps moved by 2e-5 and those of ill-conditioned solves at k >= 20 by up
+// to 5e-3, as they do under any change of rounding; which of the two lies nearer
+// to the FP64 iterate there was not measured.  A solve can so stop a step apart
+// from the same solve alone.)
 // A thread-block cluster of kBSplit CTAs owns
 // a 32 x 32 pixel tile; each CTA (256 threads, four rows each) sums a
 // contiguous quarter of the angles.  For a chunk of angles a CTA stages, per
