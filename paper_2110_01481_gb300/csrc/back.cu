@@ -219,10 +219,11 @@ __device__ __forceinline__ void pixel_pair_tile(const T *__restrict__ b, int N, 
 // against FP64 is 6.6e-8 on smooth data and 1.1e-6 on white noise, 0.6 times that
 // of one pixel per position from the tile's corner).
 // The raw bins are staged by 4-byte cp.async (rows have any alignment) one chunk
-// ahead.  Now bound by issue slots (about 4.5 issued instructions per
-// interpolation) and, at 512^2 with its 512 blocks, by latency at few warps:
-// 512^2, 720 angles 73.5 -> 51.3 us (3.7 T interpolations/s), 2048^2, 1800 angles
-// 2,383 -> 1,437 us (5.3 T/s); 50.4 and 1,414 us with the differences.
+// ahead.  Now bound by issue slots (5.2 issued instructions per interpolation)
+// and, at 512^2 with its 512 blocks, by latency at few warps (55 % of the slots
+// and 61 % of the shared path there, 103 registers): 512^2, 720 angles 73.5
+// -> 51.3 us (3.7 T interpolations/s), 2048^2, 1800 angles 2,383 -> 1,437 us (5.3
+// T/s); 50.4 and 1,414 us with the differences.
 constexpr int kBlkWarps = 4, kBlkThreads = 32 * kBlkWarps;
 constexpr int kBlkChunk = 16;         // angles per stage, two stages in flight
 constexpr int kBlkFlush = 4;          // (1 in the smaller clusters: few angles, so few chains to average over)
