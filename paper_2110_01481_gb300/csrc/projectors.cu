@@ -698,12 +698,13 @@ void launch_forward_shape(int shape, const void *pad, int N, const PadLayout &pl
     }
 }
 
-// walk range [lo, hi] of ray d of angle t, as joseph_forward_warp
-// estimates it (host arithmetic; may differ from the device's by a step).
+// walk range [lo, hi] of ray d of angle t, as joseph_forward_warp forms it, in
+// the same operations (one rounding in u0: at an angle almost parallel to the
+// walk a last bit there is the difference between no row and all of them).
 // Returns 0 for a ray that meets the image; for one that misses it (lo = N, hi
 // = -1), -1 or 1 as its crossing lies before the first or past the last row.
 int ray_range(const FwdAngle &t, int N, int d, int &lo, int &hi) {
-    const float u0 = (float)d * t.pf + t.qf;
+    const float u0 = std::fma((float)d, t.pf, t.qf);
     lo = N;
     hi = -1;
     if (std::fabs(t.df) > 1e-20f) {
@@ -836,8 +837,7 @@ void ctg_forward_plan(const FwdAngle *tab, int N, int n_angles, int n_det, const
                 }
             cost[(size_t)g * gx + bx] = (whi >= wlo ? whi - (wlo & ~3) + 1 : 0) + 16;
             if (!safe || split == 1 || pl.clamp || whi < wlo) continue;     // clamped indices are safe
-            // the device's range may differ from this estimate by a step:
-            // check a wider one
+            // the device's range, with a margin of a step of the walk's start
             const int s_lo = std::max(0, (wlo & ~3) - 4), s_hi = std::min(N - 1, whi + 4);
             // a lane's column is affine in its ray d, so the warp's first and
             // last ray of each angle are its extremes
