@@ -578,8 +578,8 @@ size_t pair_smem(int chunk, int window) {
 // CTAs per cluster for an image of `tiles` tiles: eight, halved while a CTA's
 // share would be below 30 angles (a tile's start, end and cluster sum then cost
 // as much as its angles) and the launch keeps about three CTAs per SM.  B at
-// 1024^2: 60 angles 31 us with 8, 21 with 2; 120 angles 39 and 35 (4); 2048^2, 60
-// angles 104 and 66 us.
+// 1024^2: 60 angles 29 us with 8, 23 with 2; 120 angles 37 and 35 (4); 2048^2, 60
+// angles 102 and 69 us.
 constexpr int kFullGrid = 450;
 int split_for(int n_angles, int tiles) {
     int s = kMaxSplit;
@@ -587,9 +587,10 @@ int split_for(int n_angles, int tiles) {
     return s;
 }
 // Blocks per thread of the block kernel: four (64-row tiles: half the staging
-// and parameter loads per pixel, about 7 % per row) unless the image's last tile
-// row would waste more than that or the launch would be small (512^2, 720
-// angles: 49 against 51.5 us; 700^2: 123 against 117; 361^2: 14.2 against 12.5).
+// and parameter loads per pixel, about 6 % per row) unless the image's last tile
+// row would waste more than that or the launch would be small (four against two
+// blocks: 512^2, 720 angles 48.8 against 50.1 us, 2048^2, 1800 angles 1,434 against
+// 1,533; 700^2, 720 angles 90 against 83; 361^2, 187 angles 11.7 against 11.0).
 int blocks_for(int N, int split) {
     const int rows4 = 64 * blk_tiles_y(N, 4), rows2 = 32 * blk_tiles_y(N, 2);
     return 100 * rows2 >= 93 * rows4 && back_tiles_x(N) * blk_tiles_y(N, 4) * split >= kFullGrid ? 4 : 2;
